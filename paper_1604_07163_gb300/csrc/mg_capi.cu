@@ -21,6 +21,7 @@
 #include "mg_kernels.cuh"
 #include "mg_tma.cuh"
 #include "mg_zvec.cuh"
+#include "mg_dense.cuh"
 #include "mg_g27.cuh"
 #include "mg_krylov.cuh"
 
@@ -1071,6 +1072,16 @@ mg_status unpack_level(mg_handle* h, int l, const void* src, double* dst, bool f
   return MG_OK;
 }
 
+bool overlap(const double* a, i64 na, const double* b, i64 nb) { return a < b + nb && b < a + na; }
+
+// The two dense device nodal arrays of mg_solve_host, on first use.
+mg_status host_stage(mg_handle* h) {
+  if (h->hstage[1]) return MG_OK;
+  const LevelBuf& L0 = h->lv[0];
+  for (double*& b : h->hstage) AL(b, double, (i64)L0.N[0] * L0.N[1] * L0.N[2]);
+  return MG_OK;
+}
+
 // Galerkin level l: A_l = R A_{l-1} P in float64 from the level above (its
 // 7-point edge coefficients or its 27-point couplings), then the V-cycle
 // precision copies, D^-1 and the Gershgorin bound of D^-1 A_l.
@@ -1431,6 +1442,7 @@ void release(mg_handle* h) {
   }
   if (h->vexec) cudaGraphExecDestroy(h->vexec);
   if (h->s) cudaStreamSynchronize(h->s);
+  if (h->ev_out && cudaEventSynchronize(h->ev_out) != cudaSuccess) cudaGetLastError();  // recorded inside a capture
   for (mg_handle* c : h->slab) release(c);
   for (void* p : h->allocs) cudaFree(p);
   for (cudaEvent_t e : h->evpool) cudaEventDestroy(e);
@@ -2464,12 +2476,10 @@ mg_status mg_solve_host(mg_handle* h, const double* f_host, double* x_host, doub
   const LevelBuf& L0 = h->lv[0];
   const size_t bytes = sizeof(double) * (size_t)L0.N[0] * L0.N[1] * L0.N[2];
   Guard guard(h);
-  if (!h->hstage[0]) {
-    for (double*& b : h->hstage) AL(b, double, (i64)(bytes / sizeof(double)));
-  }
+  mg_status s = host_stage(h);
+  if (s != MG_OK) return s;
   CK(cudaMemcpyAsync(h->hstage[0], f_host, bytes, cudaMemcpyHostToDevice, h->s));
   if (h->prm.nonzero_guess) CK(cudaMemcpyAsync(h->hstage[1], x_host, bytes, cudaMemcpyHostToDevice, h->s));
-  mg_status s;
   if (h->nslab > 1)
     s = dispatch(h, [&](auto impl) { return slab_solve<decltype(impl)>(h, h->hstage[0], h->hstage[1], rtol, st); });
   else if (h->prm.krylov == MG_KRYLOV_FGMRES)
@@ -2489,13 +2499,27 @@ mg_status mg_solve_host(mg_handle* h, const double* f_host, double* x_host, doub
 mg_status mg_gradient(mg_handle* h, const double* phi, const double* lambda, double* grad) {
   if (!h || !phi || !lambda || !grad) return h ? fail(h, MG_ERR_ARG, "null pointer") : MG_ERR_ARG;
   Guard guard(h);
-  mg_status s;
-  if ((s = pack_level(h, 0, phi, h->cw, true)) != MG_OK) return s;
-  if ((s = pack_level(h, 0, lambda, h->cq, true)) != MG_OK) return s;
   const LevelBuf& L0 = h->lv[0];
-  const i64 ncell = (i64)(L0.N[0] - 1) * (L0.N[1] - 1) * (L0.N[2] - 1);
-  k_gradient<<<lin_blocks(h, ncell), 256, 0, h->s>>>(L0.kc, h->cw, h->cq, L0.g, L0.ih2[0],
-                                                     L0.ih2[1], L0.ih2[2], h->prm.face_rule, grad);
+  const Geom& g = L0.g;
+  // a gradient array that overlaps an input is formed from a copy of it
+  const i64 nodes = (i64)L0.N[0] * L0.N[1] * L0.N[2], cells = (i64)(L0.N[0] - 1) * (L0.N[1] - 1) * (L0.N[2] - 1);
+  const double** in[2] = {&phi, &lambda};
+  for (int a = 0; a < 2; ++a)
+    if (overlap(*in[a], nodes, grad, cells)) {
+      mg_status s = host_stage(h);
+      if (s != MG_OK) return s;
+      CK(cudaMemcpyAsync(h->hstage[a], *in[a], sizeof(double) * nodes, cudaMemcpyDeviceToDevice, h->s));
+      *in[a] = h->hstage[a];
+    }
+  dim3 grid((g.nx + 1 + GR_TX - 1) / GR_TX, (g.ny + 1 + DN_TY - 1) / DN_TY, 1);
+  const int zs = best_zsplit(grid.x * grid.y, h->nsm * 6, g.nz + 1, 4);
+  const int kc = (g.nz + 1 + zs - 1) / zs;
+  grid.z = (g.nz + 1 + kc - 1) / kc;
+  const bool am = h->prm.face_rule != 0;
+  const double w[3] = {am ? L0.ih2[0] : 1.0 / L0.ih2[0], am ? L0.ih2[1] : 1.0 / L0.ih2[1],
+                       am ? L0.ih2[2] : 1.0 / L0.ih2[2]};
+  k_gradient<<<grid, DN_THREADS, 0, h->s>>>(L0.kc, phi, lambda, L0.kx64, L0.ky64, L0.kz64, g, w[0], w[1], w[2],
+                                            h->prm.face_rule, kc, grad);
   CKL();
   return MG_OK;
 }
@@ -2546,6 +2570,25 @@ int mg_history(const mg_handle* h, double* hist, int cap) {
 
 mg_status mg_apply(mg_handle* h, int l, const double* x, double* y) {
   if (!h || !x || !y || l < -1 || l >= h->L) return h ? fail(h, MG_ERR_ARG, "bad level or pointer") : MG_ERR_ARG;
+  // The float64 finest operator on the caller's arrays: reads only what setup
+  // wrote (setup waits for it), so it runs on the caller's stream and needs no
+  // order against the handle's own; ev_out lets mg_free wait for it.  (With the
+  // negated diagonal of test_inject 1 the product below forms its own.)
+  const LevelBuf& F = h->lv[0];
+  const i64 dense = (i64)F.N[0] * F.N[1] * F.N[2];
+  if ((l < 0 || (l == 0 && h->prm.precision == MG_FP64)) && h->prm.test_inject != 1 && !overlap(x, dense, y, dense)) {
+    const LevelBuf& L0 = F;
+    const Geom& g = L0.g;
+    dim3 grid((g.nx + 2 + DN_TX - 1) / DN_TX, (g.ny + 2 + DN_TY - 1) / DN_TY, 1);
+    const int zs = best_zsplit(grid.x * grid.y, h->nsm * 8, g.nz + 2, 2);
+    const int kc = (g.nz + 2 + zs - 1) / zs;
+    grid.z = (g.nz + 2 + kc - 1) / kc;
+    k_apply_dense<<<grid, DN_THREADS, 0, h->us>>>(x, y, L0.kx64, L0.ky64, L0.kz64, h->dg64, g, kc);
+    ++h->launches;
+    CKL();
+    CK(cudaEventRecord(h->ev_out, h->us));
+    return MG_OK;
+  }
   Guard guard(h);
   mg_status s;
   if (l < 0) {

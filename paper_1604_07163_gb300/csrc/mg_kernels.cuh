@@ -474,63 +474,6 @@ __global__ void k_combine(const double* slots, int nslab, int mode, Scal* s, int
   finish_apply(a0, a1, mode, s, flexible);
 }
 
-// ------------------------------------------------------------ gradient
-// dL/dln k_c for every finest cell from phi and lambda (padded float64):
-//   sum over the 12 edges e=(p,q) of the cell with an interior end point of
-//   -h_a^-2 (lambda_p - lambda_q)(phi_p - phi_q) * dk_e/dln k_c,
-//   dk_e/dln k_c = k_e^2/(4 k_c) (harmonic edge mean) or k_c/4 (arithmetic).
-__global__ void k_gradient(const double* __restrict__ kc, const double* __restrict__ phi,
-                           const double* __restrict__ lam, Geom g, double ihx2, double ihy2, double ihz2,
-                           int face_rule, double* __restrict__ grad) {
-  const int cx = g.nx + 1, cy = g.ny + 1, cz = g.nz + 1;
-  const i64 n = (i64)cx * cy * cz;
-  auto cell = [&](int a, int b, int c) { return kc[((i64)c * cy + b) * cx + a]; };
-  for (i64 t = blockIdx.x * (i64)blockDim.x + threadIdx.x; t < n; t += (i64)gridDim.x * blockDim.x) {
-    const int ci = (int)(t % cx);
-    const i64 r = t / cx;
-    const int cj = (int)(r % cy);
-    const int ck = (int)(r / cy);
-    const double kcv = kc[t];
-    double acc = 0.0;
-    // corner (a,b,c) of the cell is interior point (ci-1+a, cj-1+b, ck-1+c)
-    auto node = [&](const double* v, int a, int b, int c) { return v[g.at(ci - 1 + a, cj - 1 + b, ck - 1 + c)]; };
-    auto add = [&](double ke, double ih2, int a0, int b0, int c0, int a1, int b1, int c1) {
-      const double dl = node(lam, a0, b0, c0) - node(lam, a1, b1, c1);
-      const double dp = node(phi, a0, b0, c0) - node(phi, a1, b1, c1);
-      const double dke = face_rule ? 0.25 * kcv : ke * ke / (4.0 * kcv);
-      acc += -ih2 * dl * dp * dke;
-    };
-    for (int v = 0; v < 2; ++v)
-      for (int u = 0; u < 2; ++u) {
-        {  // x-edge at (J, K) = (cj+u, ck+v): needs J, K interior (full coordinates)
-          const int J = cj + u, K = ck + v;
-          if (J >= 1 && J <= g.ny && K >= 1 && K <= g.nz) {
-            const double ke = edge_mean(cell(ci, J - 1, K - 1), cell(ci, J, K - 1), cell(ci, J - 1, K),
-                                        cell(ci, J, K), face_rule);
-            add(ke, ihx2, 0, u, v, 1, u, v);
-          }
-        }
-        {  // y-edge at (I, K) = (ci+u, ck+v)
-          const int I = ci + u, K = ck + v;
-          if (I >= 1 && I <= g.nx && K >= 1 && K <= g.nz) {
-            const double ke = edge_mean(cell(I - 1, cj, K - 1), cell(I, cj, K - 1), cell(I - 1, cj, K),
-                                        cell(I, cj, K), face_rule);
-            add(ke, ihy2, u, 0, v, u, 1, v);
-          }
-        }
-        {  // z-edge at (I, J) = (ci+u, cj+v)
-          const int I = ci + u, J = cj + v;
-          if (I >= 1 && I <= g.nx && J >= 1 && J <= g.ny) {
-            const double ke = edge_mean(cell(I - 1, J - 1, ck), cell(I, J - 1, ck), cell(I - 1, J, ck),
-                                        cell(I, J, ck), face_rule);
-            add(ke, ihz2, u, v, 0, u, v, 1);
-          }
-        }
-      }
-    grad[t] = acc;
-  }
-}
-
 // ------------------------------------------------------------ telescoped bottom
 // The coarse end of the hierarchy runs inside one thread block: levels
 // lb..L-1 of the V-cycle (pre-smooth, residual, restriction down; dense
