@@ -21,6 +21,7 @@
 #include "mg_kernels.cuh"
 #include "mg_tma.cuh"
 #include "mg_zvec.cuh"
+#include "mg_bottom.cuh"
 #include "mg_dense.cuh"
 #include "mg_g27.cuh"
 #include "mg_krylov.cuh"
@@ -92,9 +93,10 @@ struct mg_handle {
   int nsm = 152;
   int L = 0, lb = 0;  // levels; first level of the bottom kernel
   int bot_cluster = 1;  // blocks of the bottom kernel (a cluster when > 1)
+  int bot_smem = 0;     // blocks of the bottom kernel in shared memory (0: it does not fit, k_bottom runs)
   LevelBuf lv[MG_MAX_LEVELS];
   double* Lc = nullptr;  // Cholesky factor of the coarsest operator
-  double* Li = nullptr;  // L^-1 and the coarsest operator inverse when that level has at most 32 unknowns
+  double* Ai = nullptr;  // inverse of the coarsest operator
   double* Ac = nullptr;  // the dense coarsest operator (inexact coarse solve)
   // flexible GMRES: basis V_0..V_m (float64), preconditioned Z_0..Z_{m-1}
   // (V-cycle precision), one column's dots and the coefficients y, partial sums
@@ -171,10 +173,11 @@ namespace {
 // One thread-block cluster of nb blocks (a bottom kernel whose passes are
 // split over nb SMs).
 template <class... KArgs, class... Args>
-void launch_cluster(const mg_handle* h, void (*kern)(KArgs...), int nb, dim3 block, Args&&... args) {
+void launch_cluster(const mg_handle* h, void (*kern)(KArgs...), int nb, dim3 block, size_t smem, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nb);
   cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = h->s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -798,12 +801,116 @@ template <class TV, class TC> struct Impl {
     return ok;
   }
 
+  // ---- bottom kernel in shared memory
+  // Fills the arguments for levels l0 .. L-1 on nb blocks (out: the buffer that
+  // receives level l0's result); returns the dynamic shared memory in bytes, 0
+  // if the levels do not fit the kernel's tables.
+  static size_t bs_args(const mg_handle* h, int l0, int nb, TV* out, BsArgs<TV, TC>* a) {
+    a->nlev = h->L - l0;
+    i64 elems = 0;
+    int planes = 0;
+    for (int l = l0; l < h->L; ++l) {
+      const LevelBuf& Lv = h->lv[l];
+      BsLevel<TV, TC>& B = a->lv[l - l0];
+      const bool last = l == h->L - 1;
+      B.g = Lv.g;
+      B.dinv = V(Lv.dinv);
+      B.dg = Lv.g27 ? V(Lv.dg) : nullptr;
+      B.kx = C(Lv.kx);
+      B.ky = C(Lv.ky);
+      B.kz = C(Lv.kz);
+      B.w = Lv.g27 ? C(Lv.w) : nullptr;
+      double it, c1[BOT_MAXDEG], c2[BOT_MAXDEG];
+      cheb_table(h->prm, Lv.beta, Lv.alpha, &it, c1, c2);
+      B.inv_theta = (TV)it;
+      for (int j = 0; j < h->prm.cheby_degree; ++j) {
+        B.c1[j] = (TV)c1[j];
+        B.c2[j] = (TV)c2[j];
+      }
+      int np = 0;  // planes of the largest block
+      for (int s = 0; s <= nb; ++s)
+        B.z0[s] = s == nb ? Lv.g.nz : l == l0 ? (int)((i64)s * Lv.g.nz / nb) : a->lv[l - 1 - l0].z0[s] / 2;
+      for (int s = 0; s < nb; ++s) np = std::max(np, B.z0[s + 1] - B.z0[s]);
+      if (last) np = Lv.g.nz;
+      for (B.lx = 0; (1 << B.lx) < Lv.g.nx;) ++B.lx;
+      for (B.ly = 0; (1 << B.ly) < Lv.g.ny;) ++B.ly;
+      const i64 win = (np + 2) * Lv.g.sz + 2 * Lv.g.Px + 16;
+      for (int c = 0; c < 2; ++c) {
+        B.ox[c] = (int)elems;
+        elems += win;
+      }
+      B.np0 = planes;
+      planes += Lv.g.nz;
+      B.cap = last ? 0 : np << (B.lx + B.ly);
+    }
+    a->xelems = (int)elems;
+    for (int l = l0; l + 1 < h->L; ++l) {
+      BsLevel<TV, TC>& B = a->lv[l - l0];
+      B.own = (int)elems;
+      elems += (i64)B.cap * (B.w ? 30 : 10);
+    }
+    if (planes > BS_PLANES || elems > (i64)1 << 20) return 0;
+    a->nu_pre = h->prm.nu_pre;
+    a->nu_post = h->prm.nu_post;
+    a->degree = h->prm.cheby_degree;
+    a->b = V(h->lv[l0].b);
+    a->out = out;
+    a->Ai = h->Ai;
+    a->Ac = h->prm.coarse_solve == 1 ? h->Ac : nullptr;
+    a->coarse_rtol = h->prm.coarse_rtol;
+    a->coarse_maxit = h->prm.coarse_maxit;
+    a->nc = h->nc;
+    return (size_t)elems * sizeof(TV);
+  }
+
+  // Whether the bottom levels fit nb blocks of the shared-memory kernel; allows it the memory it needs.
+  template <bool CL> static bool bs_fits(mg_handle* h, int nb) {
+    BsArgs<TV, TC> a{};
+    const size_t smem = bs_args(h, h->lb, nb, nullptr, &a);
+    if (smem == 0) return false;
+    cudaFuncAttributes fa;
+    int dev = 0, most = 0;
+    bool ok = cudaGetDevice(&dev) == cudaSuccess &&
+              cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
+              cudaFuncGetAttributes(&fa, k_bottom_s<TV, TC, CL>) == cudaSuccess && smem + fa.sharedSizeBytes <= (size_t)most &&
+              cudaFuncSetAttribute(k_bottom_s<TV, TC, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   most - (int)fa.sharedSizeBytes) == cudaSuccess;
+    if (ok && CL) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(nb);
+      cfg.blockDim = dim3(BS_THREADS);
+      cfg.dynamicSmemBytes = smem;
+      cudaLaunchAttribute at;
+      at.id = cudaLaunchAttributeClusterDimension;
+      at.val.clusterDim.x = nb;
+      at.val.clusterDim.y = 1;
+      at.val.clusterDim.z = 1;
+      cfg.attrs = &at;
+      cfg.numAttrs = 1;
+      int n = 0;
+      ok = cudaOccupancyMaxActiveClusters(&n, k_bottom_s<TV, TC, CL>, &cfg) == cudaSuccess && n > 0;
+    }
+    cudaGetLastError();
+    return ok;
+  }
+
   static void bottom(mg_handle* h, int l0) {
     if (h->rec) {  // a slab reached the agglomeration level: the root takes over at replay
       Pass ps;
       ps.kind = Pass::AGGLOM;
       ps.level = l0;
       h->rec->push_back(ps);
+      return;
+    }
+    if (h->bot_smem > 0) {
+      BsArgs<TV, TC> a{};
+      TV* out = V(h->lv[l0].x[l0 == h->L - 1 ? 0 : level_result_cur(h->prm)]);
+      const size_t smem = bs_args(h, l0, h->bot_smem, out, &a);
+      const int e = tm_begin(h, MG_K_BOTTOM, l0);
+      if (h->bot_smem > 1) launch_cluster(h, k_bottom_s<TV, TC, true>, h->bot_smem, dim3(BS_THREADS), smem, a);
+      else launch(h, k_bottom_s<TV, TC, false>, dim3(1), dim3(BS_THREADS), smem, a);
+      ++h->launches;
+      tm_end(h, e, MG_K_BOTTOM, l0, (double)h->lv[l0].g.npts());
       return;
     }
     BotArgs<TV, TC> a{};
@@ -834,15 +941,14 @@ template <class TV, class TC> struct Impl {
     a.nu_pre = h->prm.nu_pre;
     a.nu_post = h->prm.nu_post;
     a.degree = h->prm.cheby_degree;
-    a.Lc = h->Lc;
-    a.Li = h->Li;
+    a.Ai = h->Ai;
     a.Ac = h->prm.coarse_solve == 1 ? h->Ac : nullptr;
     a.coarse_rtol = h->prm.coarse_rtol;
     a.coarse_maxit = h->prm.coarse_maxit;
     a.nc = h->nc;
     const int e = tm_begin(h, MG_K_BOTTOM, l0);
     if (h->bot_cluster > 1)
-      launch_cluster(h, k_bottom<TV, TV, TC, true>, h->bot_cluster, dim3(BOT_THREADS), a);
+      launch_cluster(h, k_bottom<TV, TV, TC, true>, h->bot_cluster, dim3(BOT_THREADS), 0, a);
     else
       launch(h, k_bottom<TV, TV, TC, false>, dim3(1), dim3(BOT_THREADS), 0, a);
     ++h->launches;
@@ -1403,6 +1509,14 @@ mg_status build_hierarchy(mg_handle* h, int Nx, int Ny, int Nz, const double* k,
       Lv.alpha = p.eig_lo_frac * Lv.beta;
     }
   }
+  // the bottom kernel in shared memory, where the levels fit it
+  {
+    const int nb = p.bottom_blocks > 0 ? p.bottom_blocks : BS_MAXB;
+    if (dispatch(h, [&](auto impl) {
+          return nb > 1 ? decltype(impl)::template bs_fits<true>(h, nb) : decltype(impl)::template bs_fits<false>(h, nb);
+        }))
+      h->bot_smem = nb;
+  }
   // coarsest operator: dense float64 assembly and Cholesky factorisation
   AL(h->Lc, double, (i64)h->nc * h->nc);
   const LevelBuf& Cv = h->lv[L - 1];
@@ -1425,11 +1539,9 @@ mg_status build_hierarchy(mg_handle* h, int Nx, int Ny, int Nz, const double* k,
   CK(cudaMemcpyAsync(&bad, h->dflag, sizeof(int), cudaMemcpyDeviceToHost, h->s));
   CK(cudaStreamSynchronize(h->s));
   if (bad) return fail(h, MG_ERR_NOT_SPD, "coarsest operator is not positive definite");
-  if (h->nc <= 32) {
-    AL(h->Li, double, 2 * (i64)h->nc * h->nc);
-    k_trinv<<<1, 32, 0, h->s>>>(h->Lc, h->Li, h->nc);
-    CKL();
-  }
+  AL(h->Ai, double, (i64)h->nc * h->nc);
+  k_coarse_inverse<<<(h->nc + 3) / 4, 128, 0, h->s>>>(h->Lc, h->Ai, h->nc);
+  CKL();
   return MG_OK;
 }
 

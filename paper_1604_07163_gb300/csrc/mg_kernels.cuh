@@ -280,43 +280,43 @@ __global__ void k_cholesky(double* A, int n, int* bad) {
     __syncthreads();
     for (int i = j + 1 + threadIdx.x; i < n; i += blockDim.x) A[(i64)i * n + j] /= piv;
     __syncthreads();
-    const i64 m = (i64)(n - j - 1);
-    for (i64 t = threadIdx.x; t < m * m; t += blockDim.x) {
-      const int ii = j + 1 + (int)(t / m), kk = j + 1 + (int)(t % m);
-      if (kk <= ii) A[(i64)ii * n + kk] -= A[(i64)ii * n + j] * A[(i64)kk * n + j];
-    }
+    for (int ii = j + 1 + (threadIdx.x >> 5); ii < n; ii += blockDim.x >> 5)  // a warp per row
+      for (int kk = j + 1 + (threadIdx.x & 31); kk <= ii; kk += 32)
+        A[(i64)ii * n + kk] -= A[(i64)ii * n + j] * A[(i64)kk * n + j];
     __syncthreads();
   }
   for (i64 t = threadIdx.x; t < (i64)n * n; t += blockDim.x)
     if (t % n > t / n) A[t] = 0.0;
 }
 
-// Coarsest operator inverse from its Cholesky factor L (n <= 32), row-major,
-// for a coarse solve that is one matrix-vector product: Li[0, n*n) receives
-// L^-1 (thread c solves L v = e_c by forward substitution, column c) and
-// Li[n*n, 2*n*n) the symmetric A^-1 = L^-T L^-1 (entry (l, c) sums
-// L^-1(m, l) L^-1(m, c) over m >= max(l, c) in increasing m, so (l, c) and
-// (c, l) are the same sum).
-__global__ void k_trinv(const double* L, double* Li, int n) {
-  const int c = threadIdx.x;
-  double* Ai = Li + (i64)n * n;
-  if (c < n)
-    for (int r = 0; r < n; ++r) {
-      double v = 0.0;
-      if (r >= c) {
-        double s = r == c ? 1.0 : 0.0;
-        for (int q = c; q < r; ++q) s -= L[(i64)r * n + q] * Li[(i64)q * n + c];
-        v = s / L[(i64)r * n + r];
-      }
-      Li[(i64)r * n + c] = v;
-    }
-  __syncthreads();
-  if (c < n)
-    for (int l = 0; l < n; ++l) {
-      double s = 0.0;
-      for (int m = l > c ? l : c; m < n; ++m) s = fma(Li[(i64)m * n + l], Li[(i64)m * n + c], s);
-      Ai[(i64)l * n + c] = s;
-    }
+// Inverse of the coarsest operator from its Cholesky factor L, so that a
+// coarse solve is one matrix-vector product: row c of Ai is A^-1 e_c, one warp
+// per row: L v = e_c by forward substitution (row sums over the lanes), then
+// L^T x = v from the last unknown up, row r of L taking x_r out of the others.
+constexpr int MG_COARSE_MAX = 1024;
+__global__ void __launch_bounds__(128) k_coarse_inverse(const double* __restrict__ L, double* __restrict__ Ai, int n) {
+  __shared__ double vs[4][MG_COARSE_MAX];
+  const int lane = threadIdx.x & 31, c = blockIdx.x * 4 + (threadIdx.x >> 5);
+  if (c >= n) return;
+  double* v = vs[threadIdx.x >> 5];
+  for (int r = lane; r < c; r += 32) v[r] = 0.0;
+  __syncwarp();
+  for (int r = c; r < n; ++r) {
+    double s = 0.0;
+    for (int q = c + lane; q < r; q += 32) s = fma(L[(i64)r * n + q], v[q], s);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) v[r] = ((r == c ? 1.0 : 0.0) - s) / L[(i64)r * n + r];
+    __syncwarp();
+  }
+  for (int r = n - 1; r >= 0; --r) {
+    const double x = v[r] / L[(i64)r * n + r];
+    __syncwarp();
+    for (int q = lane; q < r; q += 32) v[q] = fma(-L[(i64)r * n + q], x, v[q]);
+    if (lane == 0) v[r] = x;
+    __syncwarp();
+  }
+  for (int q = lane; q < n; q += 32) Ai[(i64)c * n + q] = v[q];
 }
 
 // ------------------------------------------------------------ eigenvalue estimate
@@ -504,8 +504,7 @@ template <class TV, class TC> struct BotArgs {
   BotLevel<TV, TC> lv[BOT_MAX];
   int nlev;            // levels in this kernel; the last one is the coarsest
   int nu_pre, nu_post, degree;
-  const double* Lc;    // Cholesky factor of the coarsest operator (n x n)
-  const double* Li;    // L^-1, then the operator inverse L^-T L^-1 (n <= 32), else null
+  const double* Ai;    // inverse of the coarsest operator (n x n)
   const double* Ac;    // the coarsest operator itself (inexact solve), else null
   double coarse_rtol;  // inexact solve: GMRES-Jacobi to this relative residual,
   int coarse_maxit;    // at most this many steps (<= 32)
@@ -560,10 +559,9 @@ __device__ int bot_sweep(const BotLevel<TV, TC>& L, int cur, bool zero, const Bo
   return cur;
 }
 
-// Coarsest solve x = L^-T L^-1 b in float64 with the Cholesky factor.  For
-// n <= 32 it is one product with the precomputed inverse (k_trinv): a
-// substitution is a chain of n dependent divisions and shuffles, slow on
-// GB300's float64 pipe.  Larger n substitute with the whole block.
+// Coarsest solve x = A^-1 b in float64: one product with the precomputed
+// inverse (k_coarse_inverse).  A substitution with the Cholesky factor is a
+// chain of 2n dependent steps, each a barrier of the block.
 __device__ __forceinline__ double warp_sum_d(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -574,11 +572,11 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 // GMRES with the Jacobi preconditioner on the right, classical Gram-Schmidt,
 // Givens rotations, from zero, stopped when the rotated residual norm is at
 // most rtol ||b|| or after m (<= 32) steps.  Called by all threads of one
-// block of at least 32 warps; lane i of a warp holds component i (n <= 32);
+// block of at least 8 warps; lane i of a warp holds component i (n <= 32);
 // the Krylov basis and the Hessenberg columns live in shared memory.  Per
 // step: warps 0-7 form the matrix-vector product from column groups (their
 // partial rows added in warp order), warp i forms the Gram-Schmidt
-// coefficient of basis vector i (all from the same w), and warp 0 updates w,
+// coefficients of basis vectors i, i + warps, ... (all from the same w), and warp 0 updates w,
 // normalises it and (lane 0) applies the rotations.  y holds b on entry and
 // x on exit.
 __device__ void block_gmres(const double* A, int n, double rtol, int m, double* y) {
@@ -622,9 +620,9 @@ __device__ void block_gmres(const double* A, int n, double rtol, int m, double* 
         ws[lane] = on ? w : 0.0;
       }
       __syncthreads();
-      if (wq <= j) {  // all coefficients from the same w
-        const double h = warp_sum_d(ws[lane] * Vs[wq * 32 + lane]);
-        if (lane == 0) Hs[wq * 32 + j] = h;
+      for (int i = wq; i <= j; i += blockDim.x >> 5) {  // all coefficients from the same w
+        const double h = warp_sum_d(ws[lane] * Vs[i * 32 + lane]);
+        if (lane == 0) Hs[i * 32 + j] = h;
       }
       __syncthreads();
       if (wq == 0) {
@@ -678,60 +676,57 @@ __device__ void block_gmres(const double* A, int n, double rtol, int m, double* 
   __syncthreads();
 }
 
-template <class TV>
-__device__ void bot_coarse_solve(const Geom& g, const TV* b, TV* x, const double* Lc, const double* Li, int n,
-                                 const double* Ac = nullptr, double crtol = 0.0, int cmaxit = 0) {
-  __shared__ double y[1024];
+// y = A^-1 y for n <= 32 by a block of at least 8 warps: warp q < 8 sums
+// columns q, q + 8, q + 16, q + 24 (lane w forms row w; its at most four
+// matrix entries are loaded before the first multiply-add, so the chain is
+// one load latency and four float64 FMAs), then thread w adds the eight
+// partial rows pairwise.
+__device__ __forceinline__ void coarse_product_small(const double* Ai, int n, double* y) {
   __shared__ double part[8 * 32];
-  for (int u = threadIdx.x; u < n; u += blockDim.x) {
-    const int i = u % g.nx, j = (u / g.nx) % g.ny, k = u / (g.nx * g.ny);
-    y[u] = cvt<double>(b[g.at(i, j, k)]);
+  const int w = threadIdx.x & 31, q = threadIdx.x >> 5;
+  double v = 0.0;
+  if (q < 8 && w < n) {
+    double e[4];
+#pragma unroll
+    for (int s = 0; s < 4; ++s) e[s] = q + 8 * s < n ? Ai[(q + 8 * s) * n + w] : 0.0;
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+      if (q + 8 * s < n) v = fma(e[s], y[q + 8 * s], v);
   }
+  if (q < 8) part[q * 32 + w] = v;
   __syncthreads();
-  if (Ac && n <= 32) {
-    block_gmres(Ac, n, crtol, cmaxit, y);
-  } else if (n <= 32 && Li) {
-    // y = A^-1 y with the precomputed symmetric inverse: warp q < 8 sums
-    // columns q, q + 8, q + 16, q + 24 (lane w forms row w; its at most four
-    // matrix entries are loaded before the first multiply-add, so the
-    // chain is one load latency and four float64 FMAs), then thread w adds
-    // the eight partial rows in warp order.
-    const double* Ai = Li + n * n;
-    const int w = threadIdx.x & 31, q = threadIdx.x >> 5;
-    double v = 0.0;
-    if (q < 8 && w < n) {
-      double e[4];
+  if (threadIdx.x < n) {
+    double r[8];
 #pragma unroll
-      for (int s = 0; s < 4; ++s) e[s] = q + 8 * s < n ? Ai[(q + 8 * s) * n + w] : 0.0;
-#pragma unroll
-      for (int s = 0; s < 4; ++s)
-        if (q + 8 * s < n) v = fma(e[s], y[q + 8 * s], v);
-    }
-    if (q < 8) part[q * 32 + w] = v;
+    for (int u = 0; u < 8; ++u) r[u] = part[u * 32 + threadIdx.x];
+    y[threadIdx.x] = ((r[0] + r[1]) + (r[2] + r[3])) + ((r[4] + r[5]) + (r[6] + r[7]));
+  }
+}
+
+// Row r of A^-1 y by one warp, for any n (the same value on every lane).
+__device__ __forceinline__ double coarse_row(const double* __restrict__ Ai, int n, const double* y, int r) {
+  double v = 0.0;
+  for (int q = threadIdx.x & 31; q < n; q += 32) v = fma(__ldg(Ai + (i64)r * n + q), y[q], v);
+  return warp_sum_d(v);
+}
+
+template <class TV>
+__device__ void bot_coarse_solve(const Geom& g, const TV* b, TV* x, const double* Ai, int n, const double* Ac,
+                                 double crtol, int cmaxit) {
+  __shared__ double y[MG_COARSE_MAX];
+  auto at = [&](int u) { return g.at(u % g.nx, (u / g.nx) % g.ny, u / (g.nx * g.ny)); };
+  for (int u = threadIdx.x; u < n; u += blockDim.x) y[u] = cvt<double>(b[at(u)]);
+  __syncthreads();
+  if (Ac || n <= 32) {
+    if (Ac) block_gmres(Ac, n, crtol, cmaxit, y);
+    else coarse_product_small(Ai, n, y);
     __syncthreads();
-    if (threadIdx.x < n) {
-      double r = part[threadIdx.x];
-      for (int u = 1; u < 8; ++u) r += part[u * 32 + threadIdx.x];
-      y[threadIdx.x] = r;
-    }
+    for (int u = threadIdx.x; u < n; u += blockDim.x) x[at(u)] = store_as<TV>(y[u]);
   } else {
-    for (int c = 0; c < n; ++c) {
-      if (threadIdx.x == 0) y[c] /= Lc[(i64)c * n + c];
-      __syncthreads();
-      for (int i = c + 1 + threadIdx.x; i < n; i += blockDim.x) y[i] -= Lc[(i64)i * n + c] * y[c];
-      __syncthreads();
+    for (int r = threadIdx.x >> 5; r < n; r += blockDim.x >> 5) {
+      const double v = coarse_row(Ai, n, y, r);
+      if ((threadIdx.x & 31) == 0) x[at(r)] = store_as<TV>(v);
     }
-    for (int c = n - 1; c >= 0; --c) {
-      if (threadIdx.x == 0) y[c] /= Lc[(i64)c * n + c];
-      __syncthreads();
-      for (int i = threadIdx.x; i < c; i += blockDim.x) y[i] -= Lc[(i64)c * n + i] * y[c];
-      __syncthreads();
-    }
-  }
-  __syncthreads();
-  for (int u = threadIdx.x; u < n; u += blockDim.x) {
-    const int i = u % g.nx, j = (u / g.nx) % g.ny, k = u / (g.nx * g.ny);
-    x[g.at(i, j, k)] = store_as<TV>(y[u]);
   }
   __syncthreads();
 }
@@ -770,7 +765,7 @@ __global__ void __launch_bounds__(BOT_THREADS) k_bottom(const __grid_constant__ 
       block_prefetch_l2(V.kz, nc, tid0, nth);
     }
   }
-  if (a.Li) block_prefetch_l2(a.Li, 2 * (i64)a.nc * a.nc * (i64)sizeof(double), tid0, nth);
+  block_prefetch_l2(a.Ai, (i64)a.nc * a.nc * (i64)sizeof(double), tid0, nth);
   int cur[BOT_MAX];
   const int L = a.nlev;
   for (int l = 0; l < L - 1; ++l) {
@@ -795,7 +790,7 @@ __global__ void __launch_bounds__(BOT_THREADS) k_bottom(const __grid_constant__ 
   }
   // the coarsest solve in the first block; its barriers are block-local
   if (BS::rank() == 0)
-    bot_coarse_solve<TV>(a.lv[L - 1].g, a.lv[L - 1].b, a.lv[L - 1].x[0], a.Lc, a.Li, a.nc, a.Ac, a.coarse_rtol,
+    bot_coarse_solve<TV>(a.lv[L - 1].g, a.lv[L - 1].b, a.lv[L - 1].x[0], a.Ai, a.nc, a.Ac, a.coarse_rtol,
                          a.coarse_maxit);
   BS::sync();
   cur[L - 1] = 0;
