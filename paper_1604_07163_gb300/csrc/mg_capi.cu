@@ -25,6 +25,7 @@
 #include "mg_dense.cuh"
 #include "mg_g27.cuh"
 #include "mg_krylov.cuh"
+#include "mg_zsoft.cuh"
 
 using namespace mgdev;
 
@@ -123,6 +124,7 @@ struct mg_handle {
   cudaGraphExec_t vexec = nullptr;
   int vexec_zcur = 0;
   bool rz_fused = false;         // last V-cycle fused rho = b.z (OpChebStepDot) into its final step
+  bool soft = false;             // float64 stencil passes with products on the integer pipe (k_zsoft)
   bool zvec = true;              // stencil passes on the two-points-per-thread driver (k_zvec)
   int lin_grid = 0;              // largest grid of the linear (pointwise) kernels
   long long launches = 0;        // kernels launched (counted at launch sites)
@@ -412,6 +414,19 @@ dim3 zv_grid(const mg_handle* h, const Geom& g, int* kchunk) {
   return grid;
 }
 
+// Plane chunks of the integer-pipe driver: a chunk unpacks two planes more than
+// it writes, so at least ZS_CHUNK planes where that leaves two waves of blocks.
+dim3 zs_grid(const mg_handle* h, const Geom& g, int* kchunk) {
+  dim3 grid((g.nx + ZS_TX - 1) / ZS_TX, (g.ny + ZS_TY - 1) / ZS_TY, 1);
+  const int tiles = grid.x * grid.y;
+  const bool big = (long long)tiles * g.nz >= 2ll * ZS_CHUNK * h->nsm * ZS_BLOCKS;
+  const int zs = best_zsplit(tiles, h->nsm * ZS_BLOCKS, g.nz, big ? ZS_CHUNK : 1);
+  const int kc = (g.nz + zs - 1) / zs;
+  grid.z = (g.nz + kc - 1) / kc;
+  *kchunk = kc;
+  return grid;
+}
+
 // One z-marching pass of a point operation over level geometry g: stencil
 // operations, the prolongation and the restriction go to the two-points-per-
 // thread kernels unless the scalar driver was asked for (the float64 CG
@@ -486,6 +501,16 @@ int zmarch(mg_handle* h, const Geom& g, const Op& op, int cls = -1, int level = 
       ++h->launches;
       tm_end(h, e, cls, level, (double)g.npts());
       return 0;
+    }
+  }
+  if constexpr (Zs<Op>::ok) {
+    if (h->soft) {
+      dim3 grid = zs_grid(h, g, &kc);
+      const int e = cls >= 0 ? tm_begin(h, cls, level) : -1;
+      launch(h, k_zsoft<Op, RED>, grid, dim3(ZV_THREADS), 0, op, g, kc, h->partials, h->pstride);
+      ++h->launches;
+      tm_end(h, e, cls, level, (double)g.npts());
+      return grid.x * grid.y * grid.z;
     }
   }
   if constexpr (Zv<Op>::ok) {
@@ -965,9 +990,9 @@ template <class TV, class TC> struct Impl {
     } else if (Lv.g27) {
       OpResidual27<TV, TV, TV, TC> res{V(Lv.x[cur]), V(Lv.b), V(Lv.r), C(Lv.w), Lv.g.len, V(Lv.dg)};
       zmarch<false>(h, Lv.g, res, MG_K_RESID, l);
-    } else if (std::is_same<TV, double>::value && l == 0 && !h->rec && !h->sub) {
-      // float64 form, finest level: the stored float64 diagonal
-      OpResidualD<double> res{(const double*)Lv.x[cur], (const double*)Lv.b, (double*)Lv.r, h->dg64,
+    } else if (std::is_same<TV, double>::value && Lv.dg64) {
+      // float64 form: the stored float64 diagonal
+      OpResidualD<double> res{(const double*)Lv.x[cur], (const double*)Lv.b, (double*)Lv.r, Lv.dg64,
                               (const double*)Lv.kx, (const double*)Lv.ky, (const double*)Lv.kz};
       zmarch<false>(h, Lv.g, res, MG_K_RESID, l);
     } else {
@@ -1371,7 +1396,9 @@ mg_status build_hierarchy(mg_handle* h, int Nx, int Ny, int Nz, const double* k,
       int bad = 0;
       CK(cudaMemcpyAsync(&bad, h->dflag, sizeof(int), cudaMemcpyDeviceToHost, h->s));
       CK(cudaStreamSynchronize(h->s));
-      if (bad) return fail(h, MG_ERR_NONFINITE, "k must be positive and finite in every cell");
+      if (bad & 1) return fail(h, MG_ERR_NONFINITE, "k must be positive and finite in every cell");
+      // the integer-pipe products need coefficients well inside the float64 range and positive diagonals
+      h->soft = h->zvec && !bad && p.test_inject != 1;
     } else {
       const LevelBuf& F = h->lv[l - 1];
       k_coarsen_cells<<<lin_blocks(h, ncell), 256, 0, h->s>>>(F.kc, Lv.kc, Lv.N[0] - 1, Lv.N[1] - 1, Lv.N[2] - 1,
@@ -1437,6 +1464,10 @@ mg_status build_hierarchy(mg_handle* h, int Nx, int Ny, int Nz, const double* k,
         default:
           k_dinv<double, double, double><<<nbi, 256, 0, h->s>>>((double*)Lv.kx, (double*)Lv.ky, (double*)Lv.kz,
                                                                 (double*)Lv.dinv, Lv.g);
+          if (l > 0 && l < h->lb) {  // the float64 residual pass reads a stored diagonal
+            AL(Lv.dg64, double, n);
+            k_diag64<<<nbi, 256, 0, h->s>>>(Lv.kx64, Lv.ky64, Lv.kz64, Lv.dg64, Lv.g);
+          }
       }
       CKL();
     }
@@ -1466,6 +1497,7 @@ mg_status build_hierarchy(mg_handle* h, int Nx, int Ny, int Nz, const double* k,
       k_scale_strided<<<lin_blocks(h, n0), 256, 0, h->s>>>(h->dg64, -1.0, n0, 1);
       CKL();
     }
+    if (!mixed) h->lv[0].dg64 = h->dg64;
   }
   if (!mixed) h->lv[0].b = h->cr;  // the V-cycle's finest right-hand side is the CG residual
   // TMA-staged stencil kernels on the levels above the bottom kernel
@@ -1487,6 +1519,9 @@ mg_status build_hierarchy(mg_handle* h, int Nx, int Ny, int Nz, const double* k,
     dim3 gv = zv_grid(h, h->lv[0].g, &kcz);
     const int vg = gv.x * gv.y * gv.z;
     if (h->pstride < vg) h->pstride = vg;
+    dim3 gs = zs_grid(h, h->lv[0].g, &kcz);
+    const int ns = gs.x * gs.y * gs.z;
+    if (h->pstride < ns) h->pstride = ns;
   }
   if (h->pstride < h->lin_grid) h->pstride = h->lin_grid;
   if (h->lv[0].tma) {
@@ -1838,6 +1873,7 @@ mg_status build_slabs(mg_handle* h) {
     c->L = la + 1;
     c->lb = la;
     c->zvec = h->zvec;
+    c->soft = h->soft;
     c->lin_grid = h->lin_grid;
     for (int l = 0; l <= la; ++l) {
       const LevelBuf& G = h->lv[l];
@@ -1892,6 +1928,11 @@ mg_status build_slabs(mg_handle* h) {
           }
         }
         if ((st = slab_copy(&Lv.dinv, G.dinv, vb, 1)) != MG_OK) return st;
+        if (l > 0 && !G.g27) {
+          void* t = nullptr;
+          if ((st = slab_copy(&t, G.dg64, 8, 1)) != MG_OK) return st;
+          Lv.dg64 = (double*)t;
+        }
       }
       for (void** v : {&Lv.x[0], &Lv.x[1], &Lv.d, &Lv.r}) {
         st = alloc<char>(c, (char**)&q, n * (i64)vb);
@@ -1917,13 +1958,16 @@ mg_status build_slabs(mg_handle* h) {
       if (st != MG_OK) return st;
       if ((st = copy_slab_planes(hh, t, g0, h->dg64, h->lv[0].g, h->slab_z0[s], 8)) != MG_OK) return st;
       c->dg64 = (double*)t;
+      if (h->lv[0].dg64) c->lv[0].dg64 = c->dg64;
     }
     if (!mixed) c->lv[0].b = c->cr;
     // reduction scratch of the slab's largest reducing launch
     int kcz;
     dim3 gz = zm_grid(c, g0, &kcz);
     dim3 gv = zv_grid(c, g0, &kcz);
-    c->pstride = std::max((int)(gz.x * gz.y * gz.z), std::max((int)(gv.x * gv.y * gv.z), c->lin_grid));
+    dim3 gs = zs_grid(c, g0, &kcz);
+    c->pstride = std::max(std::max((int)(gz.x * gz.y * gz.z), (int)(gs.x * gs.y * gs.z)),
+                          std::max((int)(gv.x * gv.y * gv.z), c->lin_grid));
     {
       mg_status st = alloc<double>(c, &c->partials, 2 * (i64)c->pstride);
       if (st != MG_OK) return fail(h, st, c->err);
@@ -2691,11 +2735,12 @@ mg_status mg_apply(mg_handle* h, int l, const double* x, double* y) {
   if ((l < 0 || (l == 0 && h->prm.precision == MG_FP64)) && h->prm.test_inject != 1 && !overlap(x, dense, y, dense)) {
     const LevelBuf& L0 = F;
     const Geom& g = L0.g;
-    dim3 grid((g.nx + 2 + DN_TX - 1) / DN_TX, (g.ny + 2 + DN_TY - 1) / DN_TY, 1);
-    const int zs = best_zsplit(grid.x * grid.y, h->nsm * 8, g.nz + 2, 2);
-    const int kc = (g.nz + 2 + zs - 1) / zs;
-    grid.z = (g.nz + 2 + kc - 1) / kc;
-    k_apply_dense<<<grid, DN_THREADS, 0, h->us>>>(x, y, L0.kx64, L0.ky64, L0.kz64, h->dg64, g, kc);
+    dim3 grid((g.nx + DN_TX - 1) / DN_TX, (g.ny + DN_TY - 1) / DN_TY, 1);
+    const int zs = best_zsplit(grid.x * grid.y, h->nsm * 8, g.nz, 2);
+    const int kc = (g.nz + zs - 1) / zs;
+    grid.z = (g.nz + kc - 1) / kc;
+    (h->soft ? k_apply_dense<true> : k_apply_dense<false>)<<<grid, DN_THREADS, 0, h->us>>>(
+        x, y, L0.kx64, L0.ky64, L0.kz64, h->dg64, g, kc);
     ++h->launches;
     CKL();
     CK(cudaEventRecord(h->ev_out, h->us));
@@ -2706,8 +2751,12 @@ mg_status mg_apply(mg_handle* h, int l, const double* x, double* y) {
   if (l < 0) {
     const LevelBuf& L0 = h->lv[0];
     if ((s = pack_level(h, 0, x, h->cx, true)) != MG_OK) return s;
-    OpApply<double, double, double> op{h->cx, h->cq, L0.kx64, L0.ky64, L0.kz64};
-    zmarch<false>(h, L0.g, op);
+    if (h->soft) {
+      zmarch<false>(h, L0.g, OpApplyTo64<double>{h->cx, h->cq, h->dg64, L0.kx64, L0.ky64, L0.kz64});
+    } else {
+      OpApply<double, double, double> op{h->cx, h->cq, L0.kx64, L0.ky64, L0.kz64};
+      zmarch<false>(h, L0.g, op);
+    }
     CKL();
     return unpack_level(h, 0, h->cq, y, true);
   }

@@ -2,56 +2,109 @@
 // arrays directly, without a copy into the padded level layout and back.
 #pragma once
 #include "mg_device.cuh"
+#include "mg_zsoft.cuh"
 
 namespace mgdev {
 
 constexpr int DN_THREADS = 128;
 constexpr int DN_TX = 32, DN_TY = 4;
 
-// y = A x for the float64 finest operator, x and y dense nodal arrays (Nz, Ny,
-// Nx): y is written everywhere, 0 on the boundary, and boundary entries of x
-// count as 0.  The arithmetic is OpApply's, term for term, with the stored
-// float64 diagonal dg (the sum OpApply forms again at every point).
+// S of one point in float64 arithmetic, in stencil()'s order.  Not inlined: the
+// compiler would otherwise run it at every point beside the fixed-point sum and
+// select.
+__device__ __noinline__ double dense_exact(double uw, double ue, double us, double un, double um, double up,
+                                           const double* kx, const double* ky, const double* kz, int sy, int sz) {
+  double S = __ldg(kx - 1) * uw;
+  S = fma(__ldg(kx), ue, S);
+  S = fma(__ldg(ky - sy), us, S);
+  S = fma(__ldg(ky), un, S);
+  S = fma(__ldg(kz - sz), um, S);
+  return fma(__ldg(kz), up, S);
+}
+
+// y = A x for the float64 finest operator, x and y dense nodal arrays (nz + 2,
+// ny + 2, nx + 2): y is written everywhere, 0 on the boundary, and boundary
+// entries of x count as 0.  With SOFT a point's value is k_zsoft's bit for bit,
+// otherwise OpApplyTo64's; dg is the stored float64 diagonal.
 //
-// What bounds it: seven float64 operations per point on GB300's float64 pipe
-// (2 per clock and SM: 185 us at 257^3) against 48 bytes per point (118 us).
-// Measured at 257^3: 202 us a call; a copy into the padded layout, the product
-// with the diagonal summed at every point (12 operations) and a copy back took
-// 510 us (65^3, where launches count: 21 -> 14 us).
-// One thread owns a column of nodes and walks planes; the z neighbours stay in
-// registers, the others come through L1.
+// What bounds it: issue slots; its rows are not aligned, so a load takes a line
+// more than k_zsoft's.  Measured at 257^3: 183 us a call (48 bytes per point: 118 us of
+// traffic; 202 us in float64 arithmetic alone).
+// One thread owns a column of interior points and walks planes; the z
+// neighbours stay in registers, the others come through L1, and the streamed
+// arrays are prefetched into L2.  Warps with a point on the grid's x or y faces
+// mask the neighbours outside and also write the boundary entries of y next to
+// their points; the others do neither.
+template <bool SOFT, bool EDGE>
+__device__ __forceinline__ void dense_column(const double* __restrict__ x, double* __restrict__ y,
+                                             const double* __restrict__ kx, const double* __restrict__ ky,
+                                             const double* __restrict__ kz, const double* __restrict__ dg,
+                                             const Geom& g, int i, int j, int k0, int k1) {
+  const int sy = g.nx + 2, pz = (int)g.sz;
+  const unsigned sz = (unsigned)sy * (g.ny + 2);
+  unsigned q = (k0 + 1) * sz + (unsigned)((j + 1) * sy + i + 1);
+  int p = (int)g.at(i, j, k0);
+  const bool w = !EDGE || i > 0, e = !EDGE || i + 1 < g.nx, s = !EDGE || j > 0, n = !EDGE || j + 1 < g.ny;
+  double um = k0 > 0 ? __ldg(x + (q - sz)) : 0.0, uc = __ldg(x + q);
+  S64 sm = soft_unpack(um), sc = soft_unpack(uc), cm = soft_coef(__ldg(kz + p - pz));
+  for (int k = k0; k < k1; ++k, q += sz, p += pz) {
+    const bool top = k + 1 == g.nz;
+    const double* xq = x + q;
+    const double up = top ? 0.0 : __ldg(xq + sz), czp = __ldg(kz + p), d = __ldg(dg + p);
+    const double cxm = __ldg(kx + p - 1), cxp = __ldg(kx + p), cym = __ldg(ky + p - g.Px), cyp = __ldg(ky + p);
+    const double uw = w ? __ldg(xq - 1) : 0.0, ue = e ? __ldg(xq + 1) : 0.0;
+    const double us = s ? __ldg(xq - sy) : 0.0, un = n ? __ldg(xq + sy) : 0.0;
+    if (k + ZV_PF < k1) {
+      const int o = p + ZV_PF * pz;
+      pf_l2(kx + o);
+      pf_l2(ky + o);
+      pf_l2(kz + o);
+      pf_l2(dg + o);
+      pf_l2(xq + (ZV_PF + 1) * sz);
+    }
+    const S64 sp = soft_unpack(up), cp = soft_coef(czp);
+    double S;
+    if constexpr (SOFT) {
+      if (!soft_stencil(sm, sp, us, un, uw, ue, cm, cp, cym, cyp, cxm, cxp, S))
+        S = dense_exact(uw, ue, us, un, um, up, kx + p, ky + p, kz + p, g.Px, pz);
+    } else {
+      S = cxm * uw;
+      S = fma(cxp, ue, S);
+      S = fma(cym, us, S);
+      S = fma(cyp, un, S);
+      S = fma(__ldg(kz + p - pz), um, S);
+      S = fma(czp, up, S);
+    }
+    double* yq = y + q;
+    *yq = fma(d, uc, -S);
+    if (k == 0) yq[-(i64)sz] = 0.0;
+    if (top) yq[sz] = 0.0;
+    if (EDGE && !(w && e && s && n)) {
+      for (int c = k == 0 ? -1 : 0; c <= (top ? 1 : 0); ++c)
+        for (int b = s ? 0 : -1; b <= (n ? 0 : 1); ++b)
+          for (int a = w ? 0 : -1; a <= (e ? 0 : 1); ++a)
+            if (a | b) yq[c * (i64)sz + (i64)b * sy + a] = 0.0;
+    }
+    sm = sc;
+    sc = sp;
+    cm = cp;
+    um = uc;
+    uc = up;
+  }
+}
+template <bool SOFT>
 __global__ void __launch_bounds__(DN_THREADS, 8)
     k_apply_dense(const double* __restrict__ x, double* __restrict__ y, const double* __restrict__ kx,
                   const double* __restrict__ ky, const double* __restrict__ kz, const double* __restrict__ dg, Geom g,
                   int kchunk) {
-  const int I = blockIdx.x * DN_TX + (threadIdx.x & 31), J = blockIdx.y * DN_TY + (threadIdx.x >> 5);
-  const int Nx = g.nx + 2, Ny = g.ny + 2, Nz = g.nz + 2;
-  if (I >= Nx || J >= Ny) return;
-  const int K0 = blockIdx.z * kchunk, K1 = min(K0 + kchunk, Nz);
-  const i64 sy = Nx, sz = (i64)Nx * Ny;
-  i64 q = (i64)K0 * sz + (i64)J * sy + I;
-  const bool in = I >= 1 && I <= g.nx && J >= 1 && J <= g.ny;
-  const bool w = I >= 2, e = I <= g.nx - 1, s = J >= 2, n = J <= g.ny - 1;  // neighbours inside the boundary
-  int p = (int)g.at(I - 1, J - 1, K0 - 1);
-  auto at = [&](i64 o, int K) { return in && K >= 1 && K <= g.nz ? __ldg(x + o) : 0.0; };
-  double um = at(q - sz, K0 - 1), uc = at(q, K0);
-  for (int K = K0; K < K1; ++K, q += sz, p += (int)g.sz) {
-    const double up = at(q + sz, K + 1);
-    double v = 0.0;
-    if (in && K >= 1 && K <= g.nz) {
-      const double uw = w ? __ldg(x + q - 1) : 0.0, ue = e ? __ldg(x + q + 1) : 0.0;
-      const double us = s ? __ldg(x + q - sy) : 0.0, un = n ? __ldg(x + q + sy) : 0.0;
-      double S = __ldg(kx + p - 1) * uw;
-      S = fma(__ldg(kx + p), ue, S);
-      S = fma(__ldg(ky + p - g.Px), us, S);
-      S = fma(__ldg(ky + p), un, S);
-      S = fma(__ldg(kz + p - (int)g.sz), um, S);
-      S = fma(__ldg(kz + p), up, S);
-      v = fma(__ldg(dg + p), uc, -S);
-    }
-    y[q] = v;
-    um = uc;
-    uc = up;
+  const int i = blockIdx.x * DN_TX + (threadIdx.x & 31), j = blockIdx.y * DN_TY + (threadIdx.x >> 5);
+  const int k0 = blockIdx.z * kchunk, k1 = min(k0 + kchunk, g.nz);
+  if (j >= g.ny) return;  // whole warps
+  const int i1 = (blockIdx.x + 1) * DN_TX;
+  if (blockIdx.x > 0 && i1 < g.nx && j > 0 && j + 1 < g.ny) {
+    dense_column<SOFT, false>(x, y, kx, ky, kz, dg, g, i, j, k0, k1);
+  } else if (i < g.nx) {
+    dense_column<SOFT, true>(x, y, kx, ky, kz, dg, g, i, j, k0, k1);
   }
 }
 

@@ -143,12 +143,14 @@ __global__ void k_cast(const TS* __restrict__ src, TD* __restrict__ dst, i64 n) 
 }
 
 // ------------------------------------------------------------ setup
-// k (or ln k) per cell -> k, with a flag for non-positive / non-finite values.
+// k (or ln k) per cell -> k, with a flag for non-positive / non-finite values
+// (bit 0) and for values outside 2^-150 .. 2^150 (bit 1).
 __global__ void k_cells_init(double* kc, i64 n, int is_log, int* bad) {
   for (i64 t = blockIdx.x * (i64)blockDim.x + threadIdx.x; t < n; t += (i64)gridDim.x * blockDim.x) {
     double v = kc[t];
     if (is_log) v = exp(v);
     if (!(v > 0.0) || !isfinite(v)) atomicOr(bad, 1);
+    else if (!(v >= 0x1p-150 && v <= 0x1p150)) atomicOr(bad, 2);
     kc[t] = v;
   }
 }
