@@ -486,8 +486,11 @@ template <class R, class TV> void zv_xfer(mg_handle* h, const Geom& gc, const Op
   launch(h, k_restrict_v<R, TV>, grid, dim3(ZV_THREADS), 0, op, gc, kc);
 }
 template <class R, class TV> void zv_xfer(mg_handle* h, const Geom& g, const OpProlong<R, TV>& op) {
-  dim3 grid((g.nx + 255) / 256, (g.ny + 3) / 4, g.nz);
-  launch(h, k_prolong_v<R, TV>, grid, dim3(PV_THREADS), 0, op, g);
+  int lw = 0;  // as few idle lanes in x as a power of two allows
+  while (lw < 6 && 4 << lw < g.nx) ++lw;
+  const int rows = PV_THREADS >> lw, pairs = (g.ny + 1) / 2;
+  dim3 grid((g.nx + (4 << lw) - 1) / (4 << lw), (pairs + rows - 1) / rows, (g.nz + 1) / 2);
+  launch(h, k_prolong_v<R, TV>, grid, dim3(PV_THREADS), 0, op, g, lw);
 }
 
 template <bool RED, class Op>

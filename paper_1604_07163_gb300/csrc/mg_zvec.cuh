@@ -490,63 +490,92 @@ __global__ void __launch_bounds__(ZV_THREADS, ZvMinBlocks<Op>::value)
 
 // ------------------------------------------------------------ transfers
 // x += P e on the fine grid (OpProlong) without z-marching: each thread
-// updates four consecutive fine points of one row (one 16-byte access to x in
-// float32, two in float64); the twelve coarse values they draw on (coarse
-// columns 2m-1 .. 2m+1, two rows, two planes) come through L1.  A thread
-// owns one row chunk, so many independent read-modify-writes are in flight.
-// Same terms in the same order as OpProlong; each coarse column's sum is
-// formed once for the four points.
-constexpr int PV_THREADS = 256;  // 64 chunks of 4 points x 4 rows
+// updates a block of four consecutive x points, two rows and two planes, fine
+// (4m .. 4m+3, 2r, 2r+1, 2s, 2s+1), which draw on coarse columns 2m-1 .. 2m+1,
+// rows r-1, r and planes s-1, s: twelve coarse values for sixteen points.
+// Along an odd fine index both of OpProlong's two terms are the same coarse
+// value, so its sum doubles exactly: the sums are formed once per coarse
+// column without the doublings and the power of two goes into the factor
+// 1/8, which gives OpProlong's result bit for bit.
+//
+// What bounds it: x read and written and e/8 of memory traffic (float32: 22 us
+// at 257^3; 28 us with one row per thread); in float64 also 2.25 operations per
+// point on the float64 pipe (80 us; 4.25 operations and 141 us with each row
+// forming its own sums).
+constexpr int PV_THREADS = 256;
+// cw = 2^lw chunks of four points in x per block, 256 / cw row pairs
 template <class R, class TV>
-__global__ void __launch_bounds__(PV_THREADS) k_prolong_v(OpProlong<R, TV> op, Geom g) {
+__global__ void __launch_bounds__(PV_THREADS) k_prolong_v(OpProlong<R, TV> op, Geom g, int lw) {
   pdl_wait();
-  const int chunk = blockIdx.x * 64 + (threadIdx.x & 63);
-  const int j = blockIdx.y * 4 + (threadIdx.x >> 6);
-  const int k = blockIdx.z;
-  const int i = 4 * chunk;
-  if (j < g.ny && i < g.nx) {
+  const int m = (blockIdx.x << lw) + (threadIdx.x & ((1 << lw) - 1));
+  const int r = blockIdx.y * (PV_THREADS >> lw) + (threadIdx.x >> lw);
+  const int s = blockIdx.z;
+  const int i = 4 * m;
+  if (2 * r < g.ny && i < g.nx) {
     const Geom& gc = op.gc;
-    const int m = chunk;  // fine i = 4m: coarse columns 2m-1, 2m, 2m+1
-    const int jr[2] = {(j - 1) >> 1, j >> 1}, kp[2] = {(k - 1) >> 1, k >> 1};
-    R E[2][2][3];  // [plane k0/k1][row j0/j1][column 2m-1 .. 2m+1]
+    R E[2][2][3];  // [plane s-1 / s][row r-1 / r][column 2m-1 .. 2m+1]
 #pragma unroll
     for (int a = 0; a < 2; ++a)
 #pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        const i64 q = gc.at(2 * m - 1, jr[r], kp[a]);
+      for (int c = 0; c < 2; ++c) {
+        const i64 q = gc.at(2 * m - 1, r - 1 + c, s - 1 + a);
 #pragma unroll
-        for (int cc = 0; cc < 3; ++cc) E[a][r][cc] = cvt<R>(__ldg(op.e + q + cc));
+        for (int cc = 0; cc < 3; ++cc) E[a][c][cc] = cvt<R>(__ldg(op.e + q + cc));
       }
-    const i64 p = g.at(i, j, k);
-    R xv[4];
-    if constexpr (sizeof(TV) == 4) {
-      const float4 t = *reinterpret_cast<const float4*>(op.x + p);
-      xv[0] = t.x, xv[1] = t.y, xv[2] = t.z, xv[3] = t.w;
-    } else {
-      const double2 t0 = *reinterpret_cast<const double2*>(op.x + p);
-      const double2 t1 = *reinterpret_cast<const double2*>(op.x + p + 2);
-      xv[0] = t0.x, xv[1] = t0.y, xv[2] = t1.x, xv[3] = t1.y;
-    }
-    R Y[3];  // per coarse column: the two rows and two planes, in OpProlong's order
-#pragma unroll
-    for (int cc = 0; cc < 3; ++cc) Y[cc] = (E[0][0][cc] + E[1][0][cc]) + (E[0][1][cc] + E[1][1][cc]);
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      // coarse columns of fine 4m+e: i0 = (4m+e-1)>>1, i1 = (4m+e)>>1, as offsets from 2m-1
-      const int c0 = (e + 1) >> 1, c1 = (e + 2) >> 1;
-      xv[e] = fma((R)0.125, Y[c0] + Y[c1], xv[e]);
-    }
     const int nv = min(g.nx - i, 4);
-    if (nv == 4) {
-      if constexpr (sizeof(TV) == 4) {
-        *reinterpret_cast<float4*>(op.x + p) = make_float4(xv[0], xv[1], xv[2], xv[3]);
-      } else {
-        reinterpret_cast<double2*>(op.x + p)[0] = make_double2(xv[0], xv[1]);
-        reinterpret_cast<double2*>(op.x + p)[1] = make_double2(xv[2], xv[3]);
+    R xv[2][2][4];
+#pragma unroll
+    for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+      for (int jj = 0; jj < 2; ++jj) {
+        if (2 * s + kk >= g.nz || 2 * r + jj >= g.ny) continue;
+        const TV* x = op.x + g.at(i, 2 * r + jj, 2 * s + kk);
+        R(&v)[4] = xv[kk][jj];
+        if constexpr (sizeof(TV) == 4) {
+          const float4 t = *reinterpret_cast<const float4*>(x);
+          v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
+        } else {
+          const double2 t0 = *reinterpret_cast<const double2*>(x);
+          const double2 t1 = *reinterpret_cast<const double2*>(x + 2);
+          v[0] = t0.x, v[1] = t0.y, v[2] = t1.x, v[3] = t1.y;
+        }
       }
-    } else {
-      for (int e = 0; e < nv; ++e) op.x[p + e] = store_as<TV>(xv[e]);
+    R F[2][3], Y[2][2][3];  // F: the two planes' sum of a row; Y[kk][jj]: column sums without doublings
+#pragma unroll
+    for (int cc = 0; cc < 3; ++cc) {
+      F[0][cc] = E[0][0][cc] + E[1][0][cc];
+      F[1][cc] = E[0][1][cc] + E[1][1][cc];
+      Y[0][0][cc] = F[0][cc] + F[1][cc];
+      Y[0][1][cc] = F[1][cc];
+      Y[1][0][cc] = E[1][0][cc] + E[1][1][cc];
+      Y[1][1][cc] = E[1][1][cc];
     }
+#pragma unroll
+    for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+      for (int jj = 0; jj < 2; ++jj) {
+        if (2 * s + kk >= g.nz || 2 * r + jj >= g.ny) continue;
+        const R w = (R)(0.125 * (1 << (kk + jj)));
+        TV* x = op.x + g.at(i, 2 * r + jj, 2 * s + kk);
+        const R(&y)[3] = Y[kk][jj];
+        R(&v)[4] = xv[kk][jj];
+        v[0] = fma(w, y[0] + y[1], v[0]);
+        v[1] = fma((R)2 * w, y[1], v[1]);
+        v[2] = fma(w, y[1] + y[2], v[2]);
+        v[3] = fma((R)2 * w, y[2], v[3]);
+        if (nv == 4) {
+          if constexpr (sizeof(TV) == 4) {
+            *reinterpret_cast<float4*>(x) = make_float4(v[0], v[1], v[2], v[3]);
+          } else {
+            reinterpret_cast<double2*>(x)[0] = make_double2(v[0], v[1]);
+            reinterpret_cast<double2*>(x)[1] = make_double2(v[2], v[3]);
+          }
+        } else {
+#pragma unroll
+          for (int e = 0; e < 3; ++e)
+            if (e < nv) x[e] = store_as<TV>(v[e]);
+        }
+      }
   }
   pdl_trigger();
 }
@@ -555,7 +584,10 @@ __global__ void __launch_bounds__(PV_THREADS) k_prolong_v(OpProlong<R, TV> op, G
 // thread: the five fine values 2c .. 2c+4 of a fine row come from one
 // 16-byte load and the right lane's first value.  Per fine plane the three
 // fine rows give the plane sum; consecutive coarse planes share a fine plane,
-// whose sum is kept.  Same terms in the same order as OpRestrict.
+// whose sum is kept.  Same terms in the same order as OpRestrict, with weights
+// (1, 2, 1) per axis and the factor 1/64 at the end: powers of two, so the
+// result is the same and a coarse point takes 19 operations instead of 27,
+// which is what bounds the float64 form (257^3: 91 us, before 127 us).
 template <class R, class TV>
 __global__ void __launch_bounds__(ZV_THREADS, 8) k_restrict_v(OpRestrict<R, TV> op, Geom gc, int kchunk) {
   pdl_wait();
@@ -587,15 +619,11 @@ __global__ void __launch_bounds__(ZV_THREADS, 8) k_restrict_v(OpRestrict<R, TV> 
         if (lane == 31) v[4] = cvt<R>(__ldg(op.r + q + 4));
 #pragma unroll
         for (int e = 0; e < 2; ++e)
-          row[b][e] = fma((R)0.5, v[2 * e + 1], (R)0.25 * (v[2 * e] + v[2 * e + 2]));
+          row[b][e] = fma((R)2, v[2 * e + 1], v[2 * e] + v[2 * e + 2]);
       }
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
-        R pl = 0;
-        pl = fma((R)0.25, row[0][e], pl);
-        pl = fma((R)0.5, row[1][e], pl);
-        pl = fma((R)0.25, row[2][e], pl);
-        P[e] = pl;
+        P[e] = fma((R)2, row[1][e], row[0][e]) + row[2][e];
       }
     };
     R Plo[2], Pmid[2], Phi[2];
@@ -613,11 +641,7 @@ __global__ void __launch_bounds__(ZV_THREADS, 8) k_restrict_v(OpRestrict<R, TV> 
       R acc[2];
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
-        R a = 0;
-        a = fma((R)0.25, Plo[e], a);
-        a = fma((R)0.5, Pmid[e], a);
-        a = fma((R)0.25, Phi[e], a);
-        acc[e] = a;
+        acc[e] = (R)0.015625 * (fma((R)2, Pmid[e], Plo[e]) + Phi[e]);
       }
       if (nv > 0) st2(op.bc + gc.at(min(c, gc.Px - 2), cj, k), acc, nv);
 #pragma unroll
