@@ -24,6 +24,7 @@
 #include "mg_bottom.cuh"
 #include "mg_dense.cuh"
 #include "mg_g27.cuh"
+#include "mg_g27v.cuh"
 #include "mg_krylov.cuh"
 #include "mg_zsoft.cuh"
 
@@ -521,6 +522,24 @@ int zmarch(mg_handle* h, const Geom& g, const Op& op, int cls = -1, int level = 
       dim3 grid = zv_grid(h, g, &kc);
       const int e = cls >= 0 ? tm_begin(h, cls, level) : -1;
       launch(h, k_zvec<Op, RED>, grid, dim3(ZV_THREADS), 0, op, g, kc, h->partials, h->pstride);
+      ++h->launches;
+      tm_end(h, e, cls, level, (double)g.npts());
+      return grid.x * grid.y * grid.z;
+    }
+  }
+  if constexpr (!RED && G27<Op>::ok) {
+    if (h->zvec) {
+      constexpr int NP = GV_NP<typename G27<Op>::R>;
+      int lw = 0;  // lanes per row: a power of two up to a warp
+      while (lw < 5 && NP << lw < g.nx) ++lw;
+      const int rows = GV_THREADS >> lw;
+      dim3 grid((g.nx + (NP << lw) - 1) / (NP << lw), (g.ny + rows - 1) / rows, 1);
+      const bool big = 13.0 * sizeof(typename G27<Op>::TC) * g.npts() > 192e6;  // the couplings exceed L2
+      const int zs = best_zsplit(grid.x * grid.y, h->nsm * (big ? GV_BLOCKS<true> : GV_BLOCKS<false>), g.nz, 1);
+      kc = (g.nz + zs - 1) / zs;
+      grid.z = (g.nz + kc - 1) / kc;
+      const int e = cls >= 0 ? tm_begin(h, cls, level) : -1;
+      launch(h, big ? k_g27v<Op, NP, true> : k_g27v<Op, NP, false>, grid, dim3(GV_THREADS), 0, op, g, lw, kc);
       ++h->launches;
       tm_end(h, e, cls, level, (double)g.npts());
       return grid.x * grid.y * grid.z;

@@ -1,4 +1,4 @@
-"""The vector kernels of the transfers give the
+"""The vector kernels of the transfers and of the 27-point passes give the
 one-point-per-thread kernels' results bit for bit: rows that end inside a
 vector, rows wider than a warp's, level sizes down to three points."""
 import numpy as np
@@ -35,3 +35,16 @@ def test_transfers(gpu_lib, dims, precision):
         # the restriction alone: with x = 0 the residual is b in either kernel
         z = torch.zeros_like(x)
         assert torch.equal(A.residual_restrict(b, z, l), B.residual_restrict(b, z, l))
+
+
+@pytest.mark.parametrize("dims", DIMS)
+@pytest.mark.parametrize("precision", ["fp64", "mixed_fp32", "mixed_bf16k"])
+@pytest.mark.parametrize("degree", [2, 3])
+def test_27_point_passes(gpu_lib, dims, precision, degree):
+    A, B = pair(gpu_lib, dims, precision=precision, coarse_op="galerkin", cheby_degree=degree)
+    for l in range(1, A.num_levels):
+        b, x = (T(mi.random_nodal(A.level_shape(l), 71 + i)) for i in range(2))
+        assert torch.equal(A.smooth(b, None, l), B.smooth(b, None, l))
+        assert torch.equal(A.smooth(b, x, l), B.smooth(b, x, l))
+        if l + 1 < A.num_levels:
+            assert torch.equal(A.residual_restrict(b, x, l), B.residual_restrict(b, x, l))
