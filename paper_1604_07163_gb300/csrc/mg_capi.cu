@@ -126,7 +126,7 @@ struct mg_handle {
   int vexec_zcur = 0;
   bool rz_fused = false;         // last V-cycle fused rho = b.z (OpChebStepDot) into its final step
   bool soft = false;             // float64 stencil passes with products on the integer pipe (k_zsoft)
-  bool zvec = true;              // stencil passes on the two-points-per-thread driver (k_zvec)
+  bool zvec = true;              // stencil passes on the vector drivers (k_zvec, k_zsoft, k_g27v)
   int lin_grid = 0;              // largest grid of the linear (pointwise) kernels
   long long launches = 0;        // kernels launched (counted at launch sites)
   long long graph_launches = 0;  // kernels inside the captured V-cycle graph
@@ -428,10 +428,30 @@ dim3 zs_grid(const mg_handle* h, const Geom& g, int* kchunk) {
   return grid;
 }
 
-// One z-marching pass of a point operation over level geometry g: stencil
-// operations, the prolongation and the restriction go to the two-points-per-
-// thread kernels unless the scalar driver was asked for (the float64 CG
-// operator and the 27-point operators always use the scalar driver).
+// Launch geometry of the vector drivers, np points per thread: 2^lw lanes per
+// row, the smallest power of two up to a warp that covers it, and plane chunks
+// by wave efficiency over `blocks` resident blocks per SM, of at least `least`
+// planes where that leaves two waves of blocks (k_zvec reads two planes more
+// than it writes: at 257^3 chunks of 3 planes took 121 us a step, of 9 82 us).
+dim3 vec_grid(const mg_handle* h, const Geom& g, int np, int blocks, int least, int* lw, int* kchunk) {
+  int w = 0;
+  while (w < 5 && np << w < g.nx) ++w;
+  const int rows = ZV_THREADS >> w;
+  dim3 grid((g.nx + (np << w) - 1) / (np << w), (g.ny + rows - 1) / rows, 1);
+  const int tiles = grid.x * grid.y;
+  const bool big = (long long)tiles * g.nz >= 2ll * least * h->nsm * blocks;
+  const int zs = best_zsplit(tiles, h->nsm * blocks, g.nz, big ? least : 1);
+  const int kc = (g.nz + zs - 1) / zs;
+  grid.z = (g.nz + kc - 1) / kc;
+  *lw = w;
+  *kchunk = kc;
+  return grid;
+}
+
+// One z-marching pass of a point operation over level geometry g: the float64
+// passes go to the integer-pipe driver, other stencil operations, the 27-point
+// passes, the prolongation and the restriction to the vector kernels, unless
+// the scalar driver was asked for.
 
 // The operand of a stencil or transfer pass whose z neighbours (the pad
 // planes, which hold the neighbours' planes in a z-slab) it reads; pointwise
@@ -519,9 +539,10 @@ int zmarch(mg_handle* h, const Geom& g, const Op& op, int cls = -1, int level = 
   }
   if constexpr (Zv<Op>::ok) {
     if (h->zvec) {
-      dim3 grid = zv_grid(h, g, &kc);
+      int lw;
+      dim3 grid = vec_grid(h, g, Zv<Op>::NP, ZV_BLOCKS, ZV_CHUNK, &lw, &kc);
       const int e = cls >= 0 ? tm_begin(h, cls, level) : -1;
-      launch(h, k_zvec<Op, RED>, grid, dim3(ZV_THREADS), 0, op, g, kc, h->partials, h->pstride);
+      launch(h, k_zvec<Op, RED>, grid, dim3(ZV_THREADS), 0, op, g, lw, kc, h->partials, h->pstride);
       ++h->launches;
       tm_end(h, e, cls, level, (double)g.npts());
       return grid.x * grid.y * grid.z;
@@ -530,16 +551,11 @@ int zmarch(mg_handle* h, const Geom& g, const Op& op, int cls = -1, int level = 
   if constexpr (!RED && G27<Op>::ok) {
     if (h->zvec) {
       constexpr int NP = GV_NP<typename G27<Op>::R>;
-      int lw = 0;  // lanes per row: a power of two up to a warp
-      while (lw < 5 && NP << lw < g.nx) ++lw;
-      const int rows = GV_THREADS >> lw;
-      dim3 grid((g.nx + (NP << lw) - 1) / (NP << lw), (g.ny + rows - 1) / rows, 1);
       const bool big = 13.0 * sizeof(typename G27<Op>::TC) * g.npts() > 192e6;  // the couplings exceed L2
-      const int zs = best_zsplit(grid.x * grid.y, h->nsm * (big ? GV_BLOCKS<true> : GV_BLOCKS<false>), g.nz, 1);
-      kc = (g.nz + zs - 1) / zs;
-      grid.z = (g.nz + kc - 1) / kc;
+      int lw;
+      dim3 grid = vec_grid(h, g, NP, big ? GV_BLOCKS<true> : GV_BLOCKS<false>, 1, &lw, &kc);
       const int e = cls >= 0 ? tm_begin(h, cls, level) : -1;
-      launch(h, big ? k_g27v<Op, NP, true> : k_g27v<Op, NP, false>, grid, dim3(GV_THREADS), 0, op, g, lw, kc);
+      launch(h, big ? k_g27v<Op, NP, true> : k_g27v<Op, NP, false>, grid, dim3(ZV_THREADS), 0, op, g, lw, kc);
       ++h->launches;
       tm_end(h, e, cls, level, (double)g.npts());
       return grid.x * grid.y * grid.z;
@@ -1538,9 +1554,12 @@ mg_status build_hierarchy(mg_handle* h, int Nx, int Ny, int Nz, const double* k,
   h->lin_grid = h->nsm * (2048 / LIN_THREADS);
   h->pstride = gz.x * gz.y * gz.z;
   {
-    dim3 gv = zv_grid(h, h->lv[0].g, &kcz);
-    const int vg = gv.x * gv.y * gv.z;
-    if (h->pstride < vg) h->pstride = vg;
+    int lwz;
+    for (int np : {2, 4}) {
+      dim3 gv = vec_grid(h, h->lv[0].g, np, ZV_BLOCKS, ZV_CHUNK, &lwz, &kcz);
+      const int vg = gv.x * gv.y * gv.z;
+      if (h->pstride < vg) h->pstride = vg;
+    }
     dim3 gs = zs_grid(h, h->lv[0].g, &kcz);
     const int ns = gs.x * gs.y * gs.z;
     if (h->pstride < ns) h->pstride = ns;
@@ -1986,10 +2005,13 @@ mg_status build_slabs(mg_handle* h) {
     // reduction scratch of the slab's largest reducing launch
     int kcz;
     dim3 gz = zm_grid(c, g0, &kcz);
-    dim3 gv = zv_grid(c, g0, &kcz);
     dim3 gs = zs_grid(c, g0, &kcz);
-    c->pstride = std::max(std::max((int)(gz.x * gz.y * gz.z), (int)(gs.x * gs.y * gs.z)),
-                          std::max((int)(gv.x * gv.y * gv.z), c->lin_grid));
+    c->pstride = std::max(std::max((int)(gz.x * gz.y * gz.z), (int)(gs.x * gs.y * gs.z)), c->lin_grid);
+    int lwz;
+    for (int np : {2, 4}) {
+      dim3 gv = vec_grid(c, g0, np, ZV_BLOCKS, ZV_CHUNK, &lwz, &kcz);
+      c->pstride = std::max(c->pstride, (int)(gv.x * gv.y * gv.z));
+    }
     {
       mg_status st = alloc<double>(c, &c->partials, 2 * (i64)c->pstride);
       if (st != MG_OK) return fail(h, st, c->err);

@@ -19,34 +19,6 @@
 
 namespace mgdev {
 
-constexpr int GV_THREADS = 128;
-
-template <class R> __device__ __forceinline__ void ldn(const float* a, R (&v)[4]) {
-  const float4 t = __ldg(reinterpret_cast<const float4*>(a));
-  v[0] = cvt<R>(t.x), v[1] = cvt<R>(t.y), v[2] = cvt<R>(t.z), v[3] = cvt<R>(t.w);
-}
-template <class R> __device__ __forceinline__ void ldn(const __nv_bfloat16* a, R (&v)[4]) {
-  const uint2 t = __ldg(reinterpret_cast<const uint2*>(a));
-  const __nv_bfloat162 lo = *reinterpret_cast<const __nv_bfloat162*>(&t.x);
-  const __nv_bfloat162 hi = *reinterpret_cast<const __nv_bfloat162*>(&t.y);
-  v[0] = cvt<R>(lo.x), v[1] = cvt<R>(lo.y), v[2] = cvt<R>(hi.x), v[3] = cvt<R>(hi.y);
-}
-template <class R, class T> __device__ __forceinline__ void ldn(const T* a, R (&v)[2]) { ld2(a, v); }
-// the first n of the results
-template <class R, int NP> __device__ __forceinline__ void stn(float* a, const R (&v)[NP], int n) {
-  if constexpr (NP == 4) {
-    if (n >= 4) {
-      *reinterpret_cast<float4*>(a) = make_float4(v[0], v[1], v[2], v[3]);
-      return;
-    }
-#pragma unroll
-    for (int e = 0; e < 3; ++e)
-      if (e < n) a[e] = v[e];
-  } else {
-    st2(a, v, min(n, 2));
-  }
-}
-template <class R> __device__ __forceinline__ void stn(double* a, const R (&v)[2], int n) { st2(a, v, min(n, 2)); }
 
 // Per-operation hooks: w and its stride, the operand u, the point operation.
 template <class Op> struct G27 {
@@ -142,7 +114,7 @@ template <class R_, class TV, class TB, class TC_> struct G27<OpResidual27<R_, T
 };
 
 // 2^lw lanes per row of the level (whole rows in a warp, so that every shuffle
-// stays inside a row), GV_THREADS / 2^lw rows per block.  Lanes past the row
+// stays inside a row), ZV_THREADS / 2^lw rows per block.  Lanes past the row
 // read its last vector and store nothing; a point's right neighbour beyond its
 // own vector is never in such a lane.
 // points per thread: 16-byte vectors
@@ -155,14 +127,14 @@ template <class R> constexpr int GV_NP = sizeof(R) == 8 ? 2 : 4;
 template <bool BIG> constexpr int GV_BLOCKS = BIG ? 3 : 4;
 
 template <class Op, int NP, bool BIG>
-__global__ void __launch_bounds__(GV_THREADS, GV_BLOCKS<BIG>)
+__global__ void __launch_bounds__(ZV_THREADS, GV_BLOCKS<BIG>)
     k_g27v(Op op, Geom g, int lw, int kchunk) {
   using Z = G27<Op>;
   using R = typename Z::R;
   using TC = typename Z::TC;
   pdl_wait();
   const int W = 1 << lw, l = threadIdx.x & (W - 1);
-  const int i0 = ((blockIdx.x << lw) + l) * NP, j0 = blockIdx.y * (GV_THREADS >> lw) + (threadIdx.x >> lw);
+  const int i0 = ((blockIdx.x << lw) + l) * NP, j0 = blockIdx.y * (ZV_THREADS >> lw) + (threadIdx.x >> lw);
   const int i = min(i0, g.Px - NP), j = min(j0, g.ny - 1);
   const int nv = j0 < g.ny ? g.nx - i0 : 0;
   const int k0 = blockIdx.z * kchunk, k1 = min(k0 + kchunk, g.nz);

@@ -1,11 +1,10 @@
 // Vectorised z-marching driver for the stencil passes (default kernel).
 //
-// Each thread owns two consecutive x points of a (2*32) x 4 tile and walks a
-// chunk of planes.  Compared with one point per thread and all neighbours read
-// through L1, three things keep more HBM bytes in flight per SM:
-//   - the two points are read with one 8-byte (16-byte for float64) load per
-//     array, and the x neighbours come from the adjacent lanes by warp
-//     shuffles (only lanes 0 and 31 load theirs);
+// Each thread owns four (float64: two) consecutive x points of a row and walks a
+// chunk of planes:
+//   - every array row is read with 16-byte loads, and the x neighbours come from
+//     the adjacent lanes by warp shuffles (from memory at the ends of a row's
+//     lanes);
 //   - the operand's z neighbours live in a register queue (planes k-1, k, k+1),
 //     and everything read pointwise is loaded one plane ahead of its use;
 //   - every streamed array is prefetched into L2 two planes ahead.
@@ -13,6 +12,11 @@
 // mg_device.cuh, term for term and in the same order, so results are
 // bitwise identical to the one-point-per-thread kernel (only the block sums
 // of the reducing passes group terms differently).
+//
+// What bounds it (float32): memory traffic and its latency; a warp issues on
+// about 36% of the cycles.  257^3, two points per thread (115 instructions a
+// point, issuing on 60 to 68%) and four: zero-guess step 92 -> 77 us (59 us of
+// traffic), step 83 -> 82 (69), residual 68 -> 66 (59); 127^3 step 14.4 -> 12.2.
 #pragma once
 #include <type_traits>
 
@@ -50,19 +54,42 @@ template <class R> __device__ __forceinline__ void st2(double* a, const R (&v)[2
   if (n == 2) *reinterpret_cast<double2*>(a) = make_double2(store_as<double>(v[0]), store_as<double>(v[1]));
   else if (n == 1) a[0] = store_as<double>(v[0]);
 }
+// NP (2 or 4) consecutive elements
+template <class R> __device__ __forceinline__ void ldn(const float* a, R (&v)[4]) {
+  const float4 t = __ldg(reinterpret_cast<const float4*>(a));
+  v[0] = cvt<R>(t.x), v[1] = cvt<R>(t.y), v[2] = cvt<R>(t.z), v[3] = cvt<R>(t.w);
+}
+template <class R> __device__ __forceinline__ void ldn(const __nv_bfloat16* a, R (&v)[4]) {
+  const uint2 t = __ldg(reinterpret_cast<const uint2*>(a));
+  const __nv_bfloat162 lo = *reinterpret_cast<const __nv_bfloat162*>(&t.x);
+  const __nv_bfloat162 hi = *reinterpret_cast<const __nv_bfloat162*>(&t.y);
+  v[0] = cvt<R>(lo.x), v[1] = cvt<R>(lo.y), v[2] = cvt<R>(hi.x), v[3] = cvt<R>(hi.y);
+}
+template <class R, class T> __device__ __forceinline__ void ldn(const T* a, R (&v)[2]) { ld2(a, v); }
+// Stores the first n of NP results.
+template <class R> __device__ __forceinline__ void stn(float* a, const R (&v)[4], int n) {
+  if (n >= 4) {
+    *reinterpret_cast<float4*>(a) = make_float4(v[0], v[1], v[2], v[3]);
+    return;
+  }
+#pragma unroll
+  for (int e = 0; e < 3; ++e)
+    if (e < n) a[e] = v[e];
+}
+template <class R, class T> __device__ __forceinline__ void stn(T* a, const R (&v)[2], int n) { st2(a, v, min(n, 2)); }
 __device__ __forceinline__ void pf_l2(const void* a) { asm volatile("prefetch.global.L2 [%0];" ::"l"(a)); }
 
-// Stencil neighbourhood of the two points p, p+1: operand values u and edge
+// Stencil neighbourhood of a thread's NP points p, p+1, ..: operand values u and edge
 // coefficients (c_x of the edge entering point 0 comes from the left lane).
-template <class R> struct ZvNb {
+template <class R, int NP> struct ZvNb {
   R uw, ue, cxw;
-  R uc[2], um[2], up[2], us[2], un[2];
-  R cx[2], cys[2], cy[2], czm[2], cz[2];
+  R uc[NP], um[NP], up[NP], us[NP], un[NP];
+  R cx[NP], cys[NP], cy[NP], czm[NP], cz[NP];
   // S and D of stencil() for element e
   __device__ __forceinline__ R eval(int e, R& D) const {
-    const R cxm = e == 0 ? cxw : cx[0];
-    const R xw = e == 0 ? uw : uc[0];
-    const R xe = e == 1 ? ue : uc[1];
+    const R cxm = e == 0 ? cxw : cx[e > 0 ? e - 1 : 0];
+    const R xw = e == 0 ? uw : uc[e > 0 ? e - 1 : 0];
+    const R xe = e == NP - 1 ? ue : uc[e < NP - 1 ? e + 1 : e];
     D = ((cxm + cx[e]) + (cys[e] + cy[e])) + (czm[e] + cz[e]);
     R S = cxm * xw;
     S = fma(cx[e], xe, S);
@@ -75,25 +102,29 @@ template <class R> struct ZvNb {
 };
 
 // Per-operation hooks.  ok = false keeps an operation on the scalar driver.
-//   U      operand storage of two points (what the stencil is applied to)
-//   P      values read pointwise at the two points of the current plane
-//   load_u / vals / u_one   operand of two points / as values / of one point
+//   U      operand storage of NP points (what the stencil is applied to)
+//   P      values read pointwise at the NP points of the current plane
+//   load_u / vals / u_one   operand of NP points / as values / of one point
 //   load_p                  pointwise values of a plane
 //   prefetch(qp, qu)        L2 prefetch of the pointwise arrays at qp and of
 //                           the operand arrays at qu
 //   emit                    the point operation for the first nv points
+// points per thread: 16-byte vectors
+template <class R> constexpr int ZV_NP = sizeof(R) == 8 ? 2 : 4;
+
 template <class Op> struct Zv {
   static constexpr bool ok = false;
 };
 
 template <class R, class TV> struct ZvVecU {
+  static constexpr int NP = ZV_NP<R>;
   struct U {
-    R v[2];
+    R v[NP];
   };
-  static __device__ __forceinline__ void load(const TV* a, int p, U& u) { ld2(a + p, u.v); }
-  static __device__ __forceinline__ void vals(const U& u, R (&v)[2]) {
-    v[0] = u.v[0];
-    v[1] = u.v[1];
+  static __device__ __forceinline__ void load(const TV* a, int p, U& u) { ldn(a + p, u.v); }
+  static __device__ __forceinline__ void vals(const U& u, R (&v)[NP]) {
+#pragma unroll
+    for (int e = 0; e < NP; ++e) v[e] = u.v[e];
   }
   static __device__ __forceinline__ R one(const TV* a, int q) { return cvt<R>(__ldg(a + q)); }
 };
@@ -102,6 +133,7 @@ template <class R, class TV> struct ZvVecU {
 template <class R_, class TV, class TC_> struct Zv<OpApply<R_, TV, TC_>> {
   using Op = OpApply<R_, TV, TC_>;
   using R = R_;
+  static constexpr int NP = ZV_NP<R>;
   using TC = TC_;
   using UU = ZvVecU<R, TV>;
   using U = typename UU::U;
@@ -111,32 +143,33 @@ template <class R_, class TV, class TC_> struct Zv<OpApply<R_, TV, TC_>> {
   static __device__ __forceinline__ const TC* ky(const Op& o) { return o.ky; }
   static __device__ __forceinline__ const TC* kz(const Op& o) { return o.kz; }
   static __device__ __forceinline__ void load_u(const Op& o, int p, U& u) { UU::load(o.u, p, u); }
-  static __device__ __forceinline__ void vals(const Op&, const U& u, R (&v)[2]) { UU::vals(u, v); }
+  static __device__ __forceinline__ void vals(const Op&, const U& u, R (&v)[NP]) { UU::vals(u, v); }
   static __device__ __forceinline__ R u_one(const Op& o, int q) { return UU::one(o.u, q); }
   static __device__ __forceinline__ void load_p(const Op&, int, P&) {}
   static __device__ __forceinline__ void prefetch(const Op& o, int, int qu) { pf_l2(o.u + qu); }
-  static __device__ __forceinline__ void emit(const Op& o, int p, int nv, const ZvNb<R>& nb, const U&, const P&,
+  static __device__ __forceinline__ void emit(const Op& o, int p, int nv, const ZvNb<R, NP>& nb, const U&, const P&,
                                               double&, double&) {
-    R y[2];
+    R y[NP];
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
+    for (int e = 0; e < NP; ++e) {
       R D;
       const R S = nb.eval(e, D);
       y[e] = D * nb.uc[e] - S;
     }
-    st2(o.y + p, y, nv);
+    stn(o.y + p, y, nv);
   }
 };
 
 // Chebyshev step (OpChebStep): the pointwise part shared with the fused dot.
 template <class R, class TV, class TC> struct ZvStepP {
-  R b[2], d[2], di[2];
+  static constexpr int NP = ZV_NP<R>;
+  R b[NP], d[NP], di[NP];
 };
 template <class R, class TV, class TC>
 __device__ __forceinline__ void zv_step_load_p(const OpChebStep<R, TV, TC>& o, int p, ZvStepP<R, TV, TC>& P) {
-  ld2(o.b + p, P.b);
-  if (o.dprev) ld2(o.dprev + p, P.d);
-  if constexpr (sizeof(R) == 8) ld2(o.dinv + p, P.di);
+  ldn(o.b + p, P.b);
+  if (o.dprev) ldn(o.dprev + p, P.d);
+  if constexpr (sizeof(R) == 8) ldn(o.dinv + p, P.di);
 }
 template <class R, class TV, class TC>
 __device__ __forceinline__ void zv_step_prefetch(const OpChebStep<R, TV, TC>& o, int qp, int qu) {
@@ -146,12 +179,12 @@ __device__ __forceinline__ void zv_step_prefetch(const OpChebStep<R, TV, TC>& o,
   if constexpr (sizeof(R) == 8) pf_l2(o.dinv + qp);
 }
 // x_{j+1} of the two points, stored; returns them in xn
-template <class R, class TV, class TC>
-__device__ __forceinline__ void zv_step_emit(const OpChebStep<R, TV, TC>& o, int p, int nv, const ZvNb<R>& nb,
-                                             const ZvStepP<R, TV, TC>& P, R (&xn)[2]) {
-  R dn[2];
+template <class R, class TV, class TC, int NP>
+__device__ __forceinline__ void zv_step_emit(const OpChebStep<R, TV, TC>& o, int p, int nv, const ZvNb<R, NP>& nb,
+                                             const ZvStepP<R, TV, TC>& P, R (&xn)[NP]) {
+  R dn[NP];
 #pragma unroll
-  for (int e = 0; e < 2; ++e) {
+  for (int e = 0; e < NP; ++e) {
     R D;
     const R S = nb.eval(e, D);
     const R xp = nb.uc[e];
@@ -162,13 +195,14 @@ __device__ __forceinline__ void zv_step_emit(const OpChebStep<R, TV, TC>& o, int
     dn[e] = o.dprev ? fma(o.c1, P.d[e], o.c2 * s) : s * o.inv_theta;
     xn[e] = xp + dn[e];
   }
-  st2(o.xout + p, xn, nv);
-  if (o.dout) st2(o.dout + p, dn, nv);
+  stn(o.xout + p, xn, nv);
+  if (o.dout) stn(o.dout + p, dn, nv);
 }
 
 template <class R_, class TV, class TC_> struct Zv<OpChebStep<R_, TV, TC_>> {
   using Op = OpChebStep<R_, TV, TC_>;
   using R = R_;
+  static constexpr int NP = ZV_NP<R>;
   using TC = TC_;
   using UU = ZvVecU<R, TV>;
   using U = typename UU::U;
@@ -178,13 +212,13 @@ template <class R_, class TV, class TC_> struct Zv<OpChebStep<R_, TV, TC_>> {
   static __device__ __forceinline__ const TC* ky(const Op& o) { return o.ky; }
   static __device__ __forceinline__ const TC* kz(const Op& o) { return o.kz; }
   static __device__ __forceinline__ void load_u(const Op& o, int p, U& u) { UU::load(o.x, p, u); }
-  static __device__ __forceinline__ void vals(const Op&, const U& u, R (&v)[2]) { UU::vals(u, v); }
+  static __device__ __forceinline__ void vals(const Op&, const U& u, R (&v)[NP]) { UU::vals(u, v); }
   static __device__ __forceinline__ R u_one(const Op& o, int q) { return UU::one(o.x, q); }
   static __device__ __forceinline__ void load_p(const Op& o, int p, P& q) { zv_step_load_p(o, p, q); }
   static __device__ __forceinline__ void prefetch(const Op& o, int qp, int qu) { zv_step_prefetch(o, qp, qu); }
-  static __device__ __forceinline__ void emit(const Op& o, int p, int nv, const ZvNb<R>& nb, const U&, const P& q,
+  static __device__ __forceinline__ void emit(const Op& o, int p, int nv, const ZvNb<R, NP>& nb, const U&, const P& q,
                                               double&, double&) {
-    R xn[2];
+    R xn[NP];
     zv_step_emit(o, p, nv, nb, q, xn);
   }
 };
@@ -221,6 +255,7 @@ struct ZvFloatAcc<Z, std::void_t<decltype(Z::float_acc)>> : std::integral_consta
 template <class R_, class TV, class TC_> struct Zv<OpChebStepDot<R_, TV, TC_>> {
   using Op = OpChebStepDot<R_, TV, TC_>;
   using R = R_;
+  static constexpr int NP = ZV_NP<R>;
   using TC = TC_;
   using UU = ZvVecU<R, TV>;
   using U = typename UU::U;
@@ -230,24 +265,26 @@ template <class R_, class TV, class TC_> struct Zv<OpChebStepDot<R_, TV, TC_>> {
   static __device__ __forceinline__ const TC* ky(const Op& o) { return o.step.ky; }
   static __device__ __forceinline__ const TC* kz(const Op& o) { return o.step.kz; }
   static __device__ __forceinline__ void load_u(const Op& o, int p, U& u) { UU::load(o.step.x, p, u); }
-  static __device__ __forceinline__ void vals(const Op&, const U& u, R (&v)[2]) { UU::vals(u, v); }
+  static __device__ __forceinline__ void vals(const Op&, const U& u, R (&v)[NP]) { UU::vals(u, v); }
   static __device__ __forceinline__ R u_one(const Op& o, int q) { return UU::one(o.step.x, q); }
   static __device__ __forceinline__ void load_p(const Op& o, int p, P& q) { zv_step_load_p(o.step, p, q); }
   static __device__ __forceinline__ void prefetch(const Op& o, int qp, int qu) { zv_step_prefetch(o.step, qp, qu); }
   static constexpr bool float_acc = sizeof(R) == 4 && sizeof(TV) == 4;
-  static __device__ __forceinline__ void emit(const Op& o, int p, int nv, const ZvNb<R>& nb, const U&, const P& q,
+  static __device__ __forceinline__ void emit(const Op& o, int p, int nv, const ZvNb<R, NP>& nb, const U&, const P& q,
                                               double& a0, double&) {
-    R xn[2];
+    R xn[NP];
     zv_step_emit(o.step, p, nv, nb, q, xn);
-    if (nv > 0) a0 = fma(to_double(store_as<TV>(q.b[0])), to_double(store_as<TV>(xn[0])), a0);
-    if (nv > 1) a0 = fma(to_double(store_as<TV>(q.b[1])), to_double(store_as<TV>(xn[1])), a0);
+#pragma unroll
+    for (int e = 0; e < NP; ++e)
+      if (e < nv) a0 = fma(to_double(store_as<TV>(q.b[e])), to_double(store_as<TV>(xn[e])), a0);
   }
-  static __device__ __forceinline__ void emit_f(const Op& o, int p, int nv, const ZvNb<R>& nb, const U&,
+  static __device__ __forceinline__ void emit_f(const Op& o, int p, int nv, const ZvNb<R, NP>& nb, const U&,
                                                 const P& q, float& s, float& c) {
-    R xn[2];
+    R xn[NP];
     zv_step_emit(o.step, p, nv, nb, q, xn);
-    if (nv > 0) dot2_add((float)q.b[0], (float)store_as<TV>(xn[0]), s, c);
-    if (nv > 1) dot2_add((float)q.b[1], (float)store_as<TV>(xn[1]), s, c);
+#pragma unroll
+    for (int e = 0; e < NP; ++e)
+      if (e < nv) dot2_add((float)q.b[e], (float)store_as<TV>(xn[e]), s, c);
   }
 };
 
@@ -256,9 +293,10 @@ template <class R_, class TV, class TC_> struct Zv<OpChebStepDot<R_, TV, TC_>> {
 template <class R_, class TV, class TC_> struct Zv<OpChebZero<R_, TV, TC_>> {
   using Op = OpChebZero<R_, TV, TC_>;
   using R = R_;
+  static constexpr int NP = ZV_NP<R>;
   using TC = TC_;
   struct U {
-    R b[2], di[2];
+    R b[NP], di[NP];
   };
   struct P {};
   static constexpr bool ok = true;
@@ -266,12 +304,12 @@ template <class R_, class TV, class TC_> struct Zv<OpChebZero<R_, TV, TC_>> {
   static __device__ __forceinline__ const TC* ky(const Op& o) { return o.ky; }
   static __device__ __forceinline__ const TC* kz(const Op& o) { return o.kz; }
   static __device__ __forceinline__ void load_u(const Op& o, int p, U& u) {
-    ld2(o.b + p, u.b);
-    ld2(o.dinv + p, u.di);
+    ldn(o.b + p, u.b);
+    ldn(o.dinv + p, u.di);
   }
-  static __device__ __forceinline__ void vals(const Op& o, const U& u, R (&v)[2]) {
-    v[0] = o.inv_theta * (u.di[0] * u.b[0]);
-    v[1] = o.inv_theta * (u.di[1] * u.b[1]);
+  static __device__ __forceinline__ void vals(const Op& o, const U& u, R (&v)[NP]) {
+#pragma unroll
+    for (int e = 0; e < NP; ++e) v[e] = o.inv_theta * (u.di[e] * u.b[e]);
   }
   static __device__ __forceinline__ R u_one(const Op& o, int q) {
     return o.inv_theta * (cvt<R>(__ldg(o.dinv + q)) * cvt<R>(__ldg(o.b + q)));
@@ -281,11 +319,11 @@ template <class R_, class TV, class TC_> struct Zv<OpChebZero<R_, TV, TC_>> {
     pf_l2(o.b + qu);
     pf_l2(o.dinv + qu);
   }
-  static __device__ __forceinline__ void emit(const Op& o, int p, int nv, const ZvNb<R>& nb, const U& uc, const P&,
+  static __device__ __forceinline__ void emit(const Op& o, int p, int nv, const ZvNb<R, NP>& nb, const U& uc, const P&,
                                               double&, double&) {
-    R xo[2], d1[2];
+    R xo[NP], d1[NP];
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
+    for (int e = 0; e < NP; ++e) {
       R D;
       const R S = nb.eval(e, D);
       const R x1 = nb.uc[e];
@@ -293,8 +331,8 @@ template <class R_, class TV, class TC_> struct Zv<OpChebZero<R_, TV, TC_>> {
       d1[e] = fma(o.c1, x1, o.c2 * s);
       xo[e] = x1 + d1[e];
     }
-    st2(o.xout + p, xo, nv);
-    if (o.dout) st2(o.dout + p, d1, nv);
+    stn(o.xout + p, xo, nv);
+    if (o.dout) stn(o.dout + p, d1, nv);
   }
 };
 
@@ -302,36 +340,38 @@ template <class R_, class TV, class TC_> struct Zv<OpChebZero<R_, TV, TC_>> {
 template <class R_, class TV, class TB, class TC_> struct Zv<OpResidual<R_, TV, TB, TC_>> {
   using Op = OpResidual<R_, TV, TB, TC_>;
   using R = R_;
+  static constexpr int NP = ZV_NP<R>;
   using TC = TC_;
   using UU = ZvVecU<R, TV>;
   using U = typename UU::U;
   struct P {
-    R b[2];
+    R b[NP];
   };
   static constexpr bool ok = true;
   static __device__ __forceinline__ const TC* kx(const Op& o) { return o.kx; }
   static __device__ __forceinline__ const TC* ky(const Op& o) { return o.ky; }
   static __device__ __forceinline__ const TC* kz(const Op& o) { return o.kz; }
   static __device__ __forceinline__ void load_u(const Op& o, int p, U& u) { UU::load(o.x, p, u); }
-  static __device__ __forceinline__ void vals(const Op&, const U& u, R (&v)[2]) { UU::vals(u, v); }
+  static __device__ __forceinline__ void vals(const Op&, const U& u, R (&v)[NP]) { UU::vals(u, v); }
   static __device__ __forceinline__ R u_one(const Op& o, int q) { return UU::one(o.x, q); }
-  static __device__ __forceinline__ void load_p(const Op& o, int p, P& q) { ld2(o.b + p, q.b); }
+  static __device__ __forceinline__ void load_p(const Op& o, int p, P& q) { ldn(o.b + p, q.b); }
   static __device__ __forceinline__ void prefetch(const Op& o, int qp, int qu) {
     pf_l2(o.x + qu);
     pf_l2(o.b + qp);
   }
-  static __device__ __forceinline__ void emit(const Op& o, int p, int nv, const ZvNb<R>& nb, const U&, const P& q,
+  static __device__ __forceinline__ void emit(const Op& o, int p, int nv, const ZvNb<R, NP>& nb, const U&, const P& q,
                                               double& acc, double&) {
-    R rv[2];
+    R rv[NP];
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
+    for (int e = 0; e < NP; ++e) {
       R D;
       const R S = nb.eval(e, D);
       rv[e] = (q.b[e] + S) - D * nb.uc[e];
     }
-    st2(o.r + p, rv, nv);
-    if (nv > 0) acc = fma((double)rv[0], (double)rv[0], acc);
-    if (nv > 1) acc = fma((double)rv[1], (double)rv[1], acc);
+    stn(o.r + p, rv, nv);
+#pragma unroll
+    for (int e = 0; e < NP; ++e)
+      if (e < nv) acc = fma((double)rv[e], (double)rv[e], acc);
   }
 };
 
@@ -339,76 +379,78 @@ template <class R_, class TV, class TB, class TC_> struct Zv<OpResidual<R_, TV, 
 template <class TB> struct Zv<OpResidualD<TB>> {
   using Op = OpResidualD<TB>;
   using R = double;
+  static constexpr int NP = ZV_NP<R>;
   using TC = double;
   using UU = ZvVecU<double, double>;
   using U = typename UU::U;
   struct P {
-    double b[2], dg[2];
+    double b[NP], dg[NP];
   };
   static constexpr bool ok = true;
   static __device__ __forceinline__ const TC* kx(const Op& o) { return o.kx; }
   static __device__ __forceinline__ const TC* ky(const Op& o) { return o.ky; }
   static __device__ __forceinline__ const TC* kz(const Op& o) { return o.kz; }
   static __device__ __forceinline__ void load_u(const Op& o, int p, U& u) { UU::load(o.x, p, u); }
-  static __device__ __forceinline__ void vals(const Op&, const U& u, double (&v)[2]) { UU::vals(u, v); }
+  static __device__ __forceinline__ void vals(const Op&, const U& u, double (&v)[NP]) { UU::vals(u, v); }
   static __device__ __forceinline__ double u_one(const Op& o, int q) { return UU::one(o.x, q); }
   static __device__ __forceinline__ void load_p(const Op& o, int p, P& q) {
-    ld2(o.b + p, q.b);
-    ld2(o.dg + p, q.dg);
+    ldn(o.b + p, q.b);
+    ldn(o.dg + p, q.dg);
   }
   static __device__ __forceinline__ void prefetch(const Op& o, int qp, int qu) {
     pf_l2(o.x + qu);
     pf_l2(o.b + qp);
     pf_l2(o.dg + qp);
   }
-  static __device__ __forceinline__ void emit(const Op& o, int p, int nv, const ZvNb<double>& nb, const U&, const P& q,
+  static __device__ __forceinline__ void emit(const Op& o, int p, int nv, const ZvNb<double, NP>& nb, const U&, const P& q,
                                               double& acc, double&) {
-    double rv[2];
+    double rv[NP];
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
+    for (int e = 0; e < NP; ++e) {
       double D;
       const double S = nb.eval(e, D);
       rv[e] = (q.b[e] + S) - q.dg[e] * nb.uc[e];
     }
-    st2(o.r + p, rv, nv);
-    if (nv > 0) acc = fma(rv[0], rv[0], acc);
-    if (nv > 1) acc = fma(rv[1], rv[1], acc);
+    stn(o.r + p, rv, nv);
+#pragma unroll
+    for (int e = 0; e < NP; ++e)
+      if (e < nv) acc = fma(rv[e], rv[e], acc);
   }
 };
 
-// (The float64 CG operator, OpApplyPQ, stays on the scalar driver: it is bound
-// by the float64 pipe, and the scalar kernel measured 3% faster on it.)
+// (The float64 passes run here only where the integer-pipe driver, k_zsoft, does not apply.)
 
-// Resident blocks per SM requested from the compiler: 8 (64 registers per
-// thread) for float32 arithmetic, 4 for float64.
-template <class Op> struct ZvMinBlocks {
-  static constexpr int value = sizeof(typename Zv<Op>::R) == 8 ? 4 : 8;
-};
+// Resident blocks per SM requested from the compiler (96 registers per thread):
+// zero-guess step, step and residual at 257^3 with 4, 5 and 6 blocks 81 / 84 / 68,
+// 77 / 82 / 65 and 104 / 94 / 72 us.
+constexpr int ZV_BLOCKS = 5;
+constexpr int ZV_CHUNK = 8;  // least planes per block on large levels
 
-// The driver.  Rows j >= ny are whole warps and skip the loop (they still take
-// part in the block sum); lanes past the padded row read their own row's pad
-// slots and store nothing, so every shuffle has all 32 lanes.
+// The driver: 2^lw lanes per row (whole rows in a warp, so that every shuffle
+// stays inside a row), ZV_THREADS / 2^lw rows per block.  Lanes past the row
+// read its last vector and store nothing.
 template <class Op, bool RED>
-__global__ void __launch_bounds__(ZV_THREADS, ZvMinBlocks<Op>::value)
-    k_zvec(Op op, Geom g, int kchunk, double* partials, int stride) {
+__global__ void __launch_bounds__(ZV_THREADS, ZV_BLOCKS)
+    k_zvec(Op op, Geom g, int lw, int kchunk, double* partials, int stride) {
   using Z = Zv<Op>;
   using R = typename Z::R;
   using TC = typename Z::TC;
   using U = typename Z::U;
   using P = typename Z::P;
+  constexpr int NP = Z::NP;
   pdl_wait();
   op.prepare();
-  const int lane = threadIdx.x & 31;
-  const int i = blockIdx.x * ZV_TX + 2 * lane;
-  const int j = blockIdx.y * ZV_TY + (threadIdx.x >> 5);
+  const int W = 1 << lw, l = threadIdx.x & (W - 1);
+  const int i0 = ((blockIdx.x << lw) + l) * NP, j0 = blockIdx.y * (ZV_THREADS >> lw) + (threadIdx.x >> lw);
+  const int nv = j0 < g.ny ? min(max(g.nx - i0, 0), NP) : 0;
+  const bool first = l == 0, last = l == W - 1;
   const int k0 = blockIdx.z * kchunk;
   const int k1 = min(k0 + kchunk, g.nz);
   double a0 = 0.0, a1 = 0.0;
   float f0 = 0.0f, f1 = 0.0f;  // float-float accumulator (ZvFloatAcc ops)
-  if (j < g.ny) {
-    const int nv = min(max(g.nx - i, 0), 2);
+  {
     const int sz = (int)g.sz, sy = g.Px;
-    int p = (int)g.at(min(i, g.Px - 2), j, k0);
+    int p = (int)g.at(min(i0, g.Px - NP), min(j0, g.ny - 1), k0);
     const TC* kx = Z::kx(op);
     const TC* ky = Z::ky(op);
     const TC* kz = Z::kz(op);
@@ -416,18 +458,18 @@ __global__ void __launch_bounds__(ZV_THREADS, ZvMinBlocks<Op>::value)
     Z::load_u(op, p - sz, qm);
     Z::load_u(op, p, qc);
     Z::load_u(op, p + sz, qp);
-    R czm[2], nkx[2], nky[2], nkz[2];
-    ld2(kz + p - sz, czm);
-    ld2(kx + p, nkx);
-    ld2(ky + p, nky);
-    ld2(kz + p, nkz);
+    R czm[NP], nkx[NP], nky[NP], nkz[NP];
+    ldn(kz + p - sz, czm);
+    ldn(kx + p, nkx);
+    ldn(ky + p, nky);
+    ldn(kz + p, nkz);
     P pn;
     Z::load_p(op, p, pn);
     for (int k = k0; k < k1; ++k, p += sz) {
-      ZvNb<R> nb;
+      ZvNb<R, NP> nb;
       const P pc = pn;
 #pragma unroll
-      for (int e = 0; e < 2; ++e) {
+      for (int e = 0; e < NP; ++e) {
         nb.cx[e] = nkx[e];
         nb.cy[e] = nky[e];
         nb.cz[e] = nkz[e];
@@ -437,9 +479,9 @@ __global__ void __launch_bounds__(ZV_THREADS, ZvMinBlocks<Op>::value)
       if (k + 1 < k1) {  // next plane: operand two planes up, pointwise values one plane up
         Z::load_u(op, p + 2 * sz, qn);
         Z::load_p(op, p + sz, pn);
-        ld2(kx + p + sz, nkx);
-        ld2(ky + p + sz, nky);
-        ld2(kz + p + sz, nkz);
+        ldn(kx + p + sz, nkx);
+        ldn(ky + p + sz, nky);
+        ldn(kz + p + sz, nkz);
       }
       if (k + ZV_PF < k1) {
         const int q = p + ZV_PF * sz;
@@ -451,20 +493,20 @@ __global__ void __launch_bounds__(ZV_THREADS, ZvMinBlocks<Op>::value)
       U ys, yn;
       Z::load_u(op, p - sy, ys);
       Z::load_u(op, p + sy, yn);
-      ld2(ky + p - sy, nb.cys);
+      ldn(ky + p - sy, nb.cys);
       Z::vals(op, qc, nb.uc);
       Z::vals(op, qm, nb.um);
       Z::vals(op, qp, nb.up);
       Z::vals(op, ys, nb.us);
       Z::vals(op, yn, nb.un);
-      nb.uw = __shfl_up_sync(0xffffffffu, nb.uc[1], 1);
+      nb.uw = __shfl_up_sync(0xffffffffu, nb.uc[NP - 1], 1);
       nb.ue = __shfl_down_sync(0xffffffffu, nb.uc[0], 1);
-      nb.cxw = __shfl_up_sync(0xffffffffu, nb.cx[1], 1);
-      if (lane == 0) {
+      nb.cxw = __shfl_up_sync(0xffffffffu, nb.cx[NP - 1], 1);
+      if (first) {
         nb.uw = Z::u_one(op, p - 1);
         nb.cxw = cvt<R>(__ldg(kx + p - 1));
       }
-      if (lane == 31) nb.ue = Z::u_one(op, p + 2);
+      if (last) nb.ue = Z::u_one(op, p + NP);
       if (nv > 0) {
         if constexpr (ZvFloatAcc<Z>::value) Z::emit_f(op, p, nv, nb, qc, pc, f0, f1);
         else Z::emit(op, p, nv, nb, qc, pc, a0, a1);
@@ -473,7 +515,7 @@ __global__ void __launch_bounds__(ZV_THREADS, ZvMinBlocks<Op>::value)
       qc = qp;
       qp = qn;
 #pragma unroll
-      for (int e = 0; e < 2; ++e) czm[e] = nb.cz[e];
+      for (int e = 0; e < NP; ++e) czm[e] = nb.cz[e];
     }
   }
   pdl_trigger();
@@ -498,10 +540,9 @@ __global__ void __launch_bounds__(ZV_THREADS, ZvMinBlocks<Op>::value)
 // column without the doublings and the power of two goes into the factor
 // 1/8, which gives OpProlong's result bit for bit.
 //
-// What bounds it: x read and written and e/8 of memory traffic (float32: 22 us
-// at 257^3; 28 us with one row per thread); in float64 also 2.25 operations per
-// point on the float64 pipe (80 us; 4.25 operations and 141 us with each row
-// forming its own sums).
+// What bounds it: x read and written and e/8 of memory traffic; in float64,
+// 2.25 operations per point (4.25 when each fine row formed its own sums) on
+// the float64 pipe.
 constexpr int PV_THREADS = 256;
 // cw = 2^lw chunks of four points in x per block, 256 / cw row pairs
 template <class R, class TV>
@@ -587,7 +628,7 @@ __global__ void __launch_bounds__(PV_THREADS) k_prolong_v(OpProlong<R, TV> op, G
 // whose sum is kept.  Same terms in the same order as OpRestrict, with weights
 // (1, 2, 1) per axis and the factor 1/64 at the end: powers of two, so the
 // result is the same and a coarse point takes 19 operations instead of 27,
-// which is what bounds the float64 form (257^3: 91 us, before 127 us).
+// which is what bounds the float64 form.
 template <class R, class TV>
 __global__ void __launch_bounds__(ZV_THREADS, 8) k_restrict_v(OpRestrict<R, TV> op, Geom gc, int kchunk) {
   pdl_wait();
