@@ -56,6 +56,8 @@ def bytes_per_point(cls: str, v: int, c: int, degree: int = 2, fp64: bool = Fals
         "cheb_zero": 3 * v + c + (v if degree > 2 else 0),  # read b, dinv, k; write x (and d)
         "cheb_step": 4 * v + c + dinv,                    # (x+b+k+x'+d) and (x+d+b+k+z), averaged
         "resid": 3 * v + c,                               # read x, b, k; write r
+        "pair_pre": 4 * v + c,                            # read b, dinv (or x), k; write x, r
+        "pair_step": 3 * v + c,                           # read x, b, k; write z
         "restrict": 9 * v,                                # per coarse point: read 8 fine r, write 1
         "prolong": 2 * v + v / 8,                         # read x, e/8; write x
         "cg_dir": 32 + v,                                 # read z, p, x; write p, x (float64 p, x)
@@ -377,7 +379,7 @@ def run_ours(args):
             # dominant finest-level kernel class and of the smoother steps (events
             # inside the V-cycle graph slow the whole solve, so the headline steps
             # above run without them)
-            S.timing(True, classes=[dom] if dom == "cheb_step" else [dom, "cheb_step"], levels=[0])
+            S.timing(True, classes=sorted({dom, "cheb_step", "pair_step"}), levels=[0])
             for _ in range(args.steps):
                 S.solve(f, rtol, raise_on_error=False)
             torch.cuda.synchronize()
@@ -392,19 +394,7 @@ def run_ours(args):
             clocks = sampler.stop()
         if instrument:
             roofline = roofline_from(kt, form, clocks, dom, args.workload)
-            smoother = roofline_from(kt, form, clocks, "cheb_step", args.workload)
-            if roofline and roofline["bound"] == "alu":
-                # the rate of a float64 FMA-chain kernel on this GPU now, beside
-                # the peak derived from unit counts and the sampled clock: a
-                # lower bound on what the float64 pipe sustains, not its peak
-                fm = fp64_fma_peak()
-                if fm:
-                    roofline["fp64_probe_tflops"] = fm
-                    roofline["frac_of_probe"] = roofline["achieved"] / fm
-                    roofline["fp64_probe_source"] = (
-                        "mg_fp64_fma_peak: independent float64 FMA chains on every SM, fastest of 5 launches "
-                        "of about 16 ms, in this run after the timed steps; a lower bound on the float64 "
-                        "pipe's rate (the operator itself exceeds it on long launches), not a peak")
+            smoother = smoother_roofline(kt, form, clocks, args.workload)
             if gt:
                 gap_ms, gap_n, _ = gt
                 host_gap = {"us_per_iteration": 1e3 * gap_ms / gap_n, "ms_per_solve": gap_ms / args.steps,
@@ -561,10 +551,10 @@ def target_513_c1e6(args, dev, timed):
                               "true_rel_resid": st.true_rel_resid, "status": st.status,
                               "setup_s": st.setup_s}
         if form == "mixed_fp32":
-            S.timing(True, classes=["cheb_step"], levels=[0])
+            S.timing(True, classes=["cheb_step", "pair_step"], levels=[0])
             S.solve(f, spec["rtol"], raise_on_error=False)
             torch.cuda.synchronize()
-            out["smoother_roofline"] = roofline_from(S.kernel_times(), form, None, "cheb_step", name)
+            out["smoother_roofline"] = smoother_roofline(S.kernel_times(), form, None, name)
             S.timing(False)
         xs[form] = x.cpu().numpy()
         del x, outs
@@ -583,8 +573,6 @@ def target_513_c1e6(args, dev, timed):
     return out
 
 
-# float64 operations per point of the float64-pipe-bound outer-CG kernel
-# (6 FMA for the neighbour sum, 1 for D p - S, 1 for p.q)
 # Method variants timed beside the headline solve (same problem, precision and
 # tolerance): Galerkin coarse operators, and the two solver configurations of
 # the paper's Sec. 5 experiments.
@@ -594,9 +582,6 @@ VARIANTS = {
                                                      nu_pre=8, nu_post=8, coarse_solve="gmres", coarse_rtol=1e-4),
     "fgmres_rediscretised_chebyshev10": dict(krylov="fgmres", cheby_degree=10),
 }
-CG_APPLY_FLOPS = 16
-# GB300: 152 SMs x 2 float64 FMA per clock per SM (the nominal 1.25 TFLOP/s at 2.07 GHz)
-FP64_FLOP_PER_SM_CLK = 4
 
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) of the
 # finest-level kernel classes, from one ncu capture each on the 257^3 workload
@@ -659,34 +644,15 @@ def measured_traffic(workload, form, cls):
     return rec[0]
 
 
-def fp64_fma_peak(launches=5):
-    """Rate of the library's float64 FMA-chain probe on the current GPU in
-    TFLOP/s (a lower bound on the float64 pipe's rate), or None."""
-    import ctypes
-    from paper_1604_07163_gb300 import _lib
-    r = ctypes.c_double()
-    rc = _lib.load().mg_fp64_fma_peak(launches, ctypes.byref(r))
-    return r.value if rc == 0 else None
-
-
 def roofline_from(kt, form, clocks, cls, workload):
     """Roofline entry of level-0 kernel class cls from the live CUDA-event
-    timing: algorithmic GB/s vs the measured HBM peak, or float64 FLOP/s vs
-    the float64 pipe peak for the float64-pipe-bound outer-CG operator."""
+    timing: algorithmic GB/s vs the measured HBM peak."""
     rec = kt.get((cls, 0))
     if rec is None:
         return None
     ms, nl, pts = rec
     avg_s = ms * 1e-3 / nl
     traffic = measured_traffic(workload, form, cls)
-    if cls == "cg_apply":
-        mhz = clocks["sm_mhz"] if clocks else 2070.0
-        fpeak = 152 * FP64_FLOP_PER_SM_CLK * mhz * 1e6 / 1e12
-        flops = CG_APPLY_FLOPS * pts / nl
-        ach = flops / avg_s / 1e12
-        return {"bound": "alu", "kernel": cls, "achieved": ach, "peak": fpeak, "unit": "TFLOP/s",
-                "frac": ach / fpeak, "peak_source": "derived: 152 SMs x 4 float64 flop/clk x median SM clock",
-                "traffic": traffic, "algorithmic_flops_per_launch": flops, "avg_launch_ms": ms / nl, "launches": nl}
     v, c = form_sizes(form)
     peak, which = load_peaks()
     bpp = bytes_per_point(cls, v, c, fp64=form == "fp64")
@@ -695,6 +661,12 @@ def roofline_from(kt, form, clocks, cls, workload):
     return {"bound": "hbm", "kernel": cls, "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak, "peak_source": which, "traffic": traffic,
             "algorithmic_bytes_per_launch": alg, "avg_launch_ms": ms / nl, "launches": nl}
+
+
+def smoother_roofline(kt, form, clocks, workload):
+    """The finest level's smoothing steps: two to a sweep where the level runs them so, single ones otherwise."""
+    return (roofline_from(kt, form, clocks, "pair_step", workload)
+            or roofline_from(kt, form, clocks, "cheb_step", workload))
 
 
 def main():

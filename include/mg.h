@@ -344,7 +344,7 @@ mg_status mg_residual_norm_noalloc(mg_handle* h, const double* f, const double* 
  * on a level in level_mask (bit l = level l) is bracketed by CUDA events on
  * the launching stream and its device time is accumulated per class and
  * level.  class_mask = 0 disables timing.  While a class run inside the
- * V-cycle (MG_K_CHEB_ZERO .. MG_K_BOTTOM, MG_K_DOT) is timed, the V-cycle is
+ * V-cycle (MG_K_CHEB_ZERO .. MG_K_BOTTOM, MG_K_DOT, MG_K_PAIR_*) is timed, the V-cycle is
  * launched kernel by kernel (not from the graph) so that the events are plain
  * stream events; timing only other classes keeps the graph.  Enabling or
  * disabling resets the counters. */
@@ -364,7 +364,9 @@ typedef enum {
   MG_K_HOST_GAP = 11,  /* not a kernel: per outer CG iteration, the device time from the end of the
                           iteration's last kernel to the next V-cycle's launch, i.e. the read of the CG
                           scalars by the host, its convergence test and its next launch (points = 0) */
-  MG_K_NCLASS = 12
+  MG_K_PAIR_PRE = 12,  /* smoothing and the residual in one sweep: the steps from a zero guess (Chebyshev), or a step */
+  MG_K_PAIR_STEP = 13, /* two smoothing steps in one sweep */
+  MG_K_NCLASS = 14
 } mg_kernel_class;
 mg_status mg_timing_enable(mg_handle* h, int class_mask, int level_mask);
 /* Totals for class cls on level l (0 = finest): device milliseconds, number of

@@ -25,7 +25,7 @@ EXPORTS = [
     "mg_set_transport", "mg_fp64_fma_peak",
 ]
 KERNEL_CLASSES = ["cheb_zero", "cheb_step", "resid", "restrict", "prolong", "bottom", "cg_dir", "cg_upd", "dot",
-                  "cast", "cg_apply", "host_gap"]
+                  "cast", "cg_apply", "host_gap", "pair_pre", "pair_step"]
 
 
 class MgParams(C.Structure):

@@ -26,6 +26,7 @@
 #include "mg_g27.cuh"
 #include "mg_g27v.cuh"
 #include "mg_krylov.cuh"
+#include "mg_pair.cuh"
 #include "mg_zsoft.cuh"
 
 using namespace mgdev;
@@ -448,6 +449,36 @@ dim3 vec_grid(const mg_handle* h, const Geom& g, int np, int blocks, int least, 
   return grid;
 }
 
+// Launch geometry of k_pair: the lanes per row (and whether neighbouring tiles
+// share points in x) with the least work on tile rims, and plane chunks of at
+// least 12 for one block per SM.  Tiles that share points have at least 32
+// lanes, 512 bytes of a row: at 511^3 points 16 lanes have less rim (1.41 against 1.45
+// of the points) but took 1144 us instead of 1062 for two steps.
+struct PairGrid {
+  dim3 grid;
+  int lx, halo, kchunk;
+};
+PairGrid pair_grid(const mg_handle* h, const Geom& g) {
+  PairGrid b{};
+  double best = 0.0;
+  for (int lx = 2; lx <= 6; ++lx)
+    for (int halo = 0; halo < 2; ++halo) {
+      const int LX = 1 << lx, LY = PR_THREADS >> lx;
+      if (halo ? LX < 32 : PR_NP * LX < g.nx) continue;
+      const int wide = PR_NP * (LX - 2 * halo), tx = (g.nx + wide - 1) / wide, ty = (g.ny + LY - 3) / (LY - 2);
+      const double cost = (double)tx * ty;
+      if (best != 0.0 && cost >= best) continue;
+      best = cost;
+      b.grid = dim3(tx, ty, 1);
+      b.lx = lx;
+      b.halo = halo;
+    }
+  const int zs = best_zsplit(b.grid.x * b.grid.y, h->nsm, g.nz, 12);
+  b.kchunk = (g.nz + zs - 1) / zs;
+  b.grid.z = (g.nz + b.kchunk - 1) / b.kchunk;
+  return b;
+}
+
 // One z-marching pass of a point operation over level geometry g: the float64
 // passes go to the integer-pipe driver, other stencil operations, the 27-point
 // passes, the prolongation and the restriction to the vector kernels, unless
@@ -652,6 +683,12 @@ void cheb_table(const mg_params& p, double beta_l, double alpha_l, double* inv_t
 
 mg_status read_scal(mg_handle* h);
 
+// Levels from this size run their smoothing passes two to a sweep.  At 127^3 points the sweep
+// takes what its two passes do (22.3 + 22.8 us against 24.4 + 28.5 us timed singly, but a
+// 129^3 gradient step 11.8 ms against 11.4 ms: its blocks leave no room for the next
+// kernel's); at 255^3 it saves a quarter.
+constexpr double PAIR_MIN_POINTS = 4e6;
+
 template <class TV, class TC> struct Impl {
   using TVt = TV;
   using TCt = TC;
@@ -842,6 +879,7 @@ template <class TV, class TC> struct Impl {
     const mg_params& p = h->prm;
     OpProlong<TV, TV> pr{Cv.g, V(Cv.x[ccur]), V(Lv.x[cur])};
     zmarch<false>(h, Lv.g, pr, MG_K_PROLONG, l);
+    if (paired(h, l)) return pair_post(h, l, cur, fuse_rz);
     for (int s = 0; s < p.nu_post; ++s) cur = sweep(h, l, cur, false, fuse_rz && s + 1 == p.nu_post);
     return cur;
   }
@@ -1020,8 +1058,15 @@ template <class TV, class TC> struct Impl {
 
   // r = b - A x[cur] on level l, then b of level l+1 = R r.
   static void residual_restrict(mg_handle* h, int l, int cur) {
+    residual(h, l, cur);
+    restrict_residual(h, l);
+  }
+  static void restrict_residual(mg_handle* h, int l) {
+    OpRestrict<TV, TV> rs{h->lv[l].g, V(h->lv[l].r), V(h->lv[l + 1].b)};
+    zmarch<false>(h, h->lv[l + 1].g, rs, MG_K_RESTRICT, l);
+  }
+  static void residual(mg_handle* h, int l, int cur) {
     LevelBuf& Lv = h->lv[l];
-    LevelBuf& Cv = h->lv[l + 1];
     if (Lv.tma) {
       tma_launch<TK_RESID, false, false>(h, l, Lv.m_full_x[cur], nullptr, V(Lv.r), nullptr, 0.0, 0.0, 0.0,
                                          MG_K_RESID);
@@ -1037,8 +1082,66 @@ template <class TV, class TC> struct Impl {
       OpResidual<TV, TV, TV, TC> res{V(Lv.x[cur]), V(Lv.b), V(Lv.r), C(Lv.kx), C(Lv.ky), C(Lv.kz)};
       zmarch<false>(h, Lv.g, res, MG_K_RESID, l);
     }
-    OpRestrict<TV, TV> rs{Lv.g, V(Lv.r), V(Cv.b)};
-    zmarch<false>(h, Cv.g, rs, MG_K_RESTRICT, l);
+  }
+
+  // ---- two passes in one sweep (k_pair)
+  // Levels whose smoothing passes run two to a sweep: float32, 7-point, the
+  // default driver, Chebyshev(2) or Richardson.  (A z-slab's halo planes are
+  // exchanged before every single pass.)
+  static bool paired(const mg_handle* h, int l) {
+    const LevelBuf& Lv = h->lv[l];
+    const mg_params& p = h->prm;
+    return std::is_same<TV, float>::value && h->zvec && p.stencil_kernel == 0 && !h->rec && !h->sub && !Lv.g27 &&
+           !Lv.tma && (double)Lv.g.npts() >= PAIR_MIN_POINTS && p.nu_pre > 0 &&
+           (p.cheby_degree == 1 || (p.cheby_degree == 2 && p.nu_pre == 1));
+  }
+  // passes A, B from buffer cur; the iterate goes to the other buffer
+  template <int A, int B, bool DOT> static int pair(mg_handle* h, int l, int cur, int cls) {
+    if constexpr (std::is_same<TV, float>::value) {
+      LevelBuf& Lv = h->lv[l];
+      double it, c1[BOT_MAXDEG], c2[BOT_MAXDEG];
+      cheb_table(h->prm, Lv.beta, Lv.alpha, &it, c1, c2);
+      const bool two = h->prm.cheby_degree > 1;
+      PairArgs<TC> a{V(Lv.x[cur]), V(Lv.b),    V(Lv.dinv), V(Lv.x[cur ^ 1]), V(Lv.r), C(Lv.kx),
+                     C(Lv.ky),     C(Lv.kz),   two ? (float)c1[1] : 0.0f,    two ? (float)c2[1] : 0.0f,
+                     (float)it,    two ? 1 : 0};
+      const PairGrid b = pair_grid(h, Lv.g);
+      const size_t smem = sizeof(float) * 2 * (PR_THREADS >> b.lx) * (PR_NP * (1 << b.lx) + 8);
+      const int e = tm_begin(h, cls, l);
+      launch(h, k_pair<TC, A, B, DOT>, b.grid, dim3(PR_THREADS), smem, a, Lv.g, b.lx, b.halo, b.kchunk, h->partials,
+             h->pstride);
+      ++h->launches;
+      tm_end(h, e, cls, l, (double)Lv.g.npts());
+      if (DOT) {
+        finish(h, b.grid.x * b.grid.y * b.grid.z, FIN_RZ);
+        h->rz_fused = true;
+      }
+    }
+    return cur ^ 1;
+  }
+  // Pre-smoothing from a zero guess and the residual.
+  static int pair_pre(mg_handle* h, int l) {
+    if (h->prm.cheby_degree == 2) return pair<PR_ZERO, PR_RESID, false>(h, l, 0, MG_K_PAIR_PRE);
+    int cur = sweep(h, l, 0, true), m = h->prm.nu_pre - 1;
+    if (m == 0) {
+      residual(h, l, cur);
+      return cur;
+    }
+    if (m % 2 == 0) cur = sweep(h, l, cur, false), --m;
+    for (; m > 1; m -= 2) cur = pair<PR_STEP, PR_STEP, false>(h, l, cur, MG_K_PAIR_STEP);
+    return pair<PR_STEP, PR_RESID, false>(h, l, cur, MG_K_PAIR_PRE);
+  }
+  static int pair_post(mg_handle* h, int l, int cur, bool fuse_rz) {
+    const mg_params& p = h->prm;
+    int m = p.nu_post * p.cheby_degree;  // steps
+    if (m % 2) {
+      cur = sweep(h, l, cur, false, fuse_rz && m == 1);
+      --m;
+    }
+    for (; m > 0; m -= 2)
+      cur = fuse_rz && m == 2 ? pair<PR_STEP, PR_STEP, true>(h, l, cur, MG_K_PAIR_STEP)
+                              : pair<PR_STEP, PR_STEP, false>(h, l, cur, MG_K_PAIR_STEP);
+    return cur;
   }
 
   // V-cycle from level l with zero initial guess; b of level l must be set.
@@ -1050,6 +1153,11 @@ template <class TV, class TC> struct Impl {
     }
     LevelBuf& Lv = h->lv[l];
     int cur = 0;
+    if (paired(h, l)) {
+      cur = pair_pre(h, l);
+      restrict_residual(h, l);
+      return correct_and_post_smooth(h, l, cur, vcycle(h, l + 1), fuse_rz);
+    }
     for (int s = 0; s < h->prm.nu_pre; ++s) cur = sweep(h, l, cur, s == 0);
     if (h->prm.nu_pre == 0) {
       void* x0 = Lv.x[0];
@@ -1561,7 +1669,8 @@ mg_status build_hierarchy(mg_handle* h, int Nx, int Ny, int Nz, const double* k,
       if (h->pstride < vg) h->pstride = vg;
     }
     dim3 gs = zs_grid(h, h->lv[0].g, &kcz);
-    const int ns = gs.x * gs.y * gs.z;
+    const dim3 gp = pair_grid(h, h->lv[0].g).grid;
+    const int ns = std::max(gs.x * gs.y * gs.z, gp.x * gp.y * gp.z);
     if (h->pstride < ns) h->pstride = ns;
   }
   if (h->pstride < h->lin_grid) h->pstride = h->lin_grid;
@@ -1649,7 +1758,8 @@ void release(mg_handle* h) {
 
 // kernel classes launched inside the V-cycle (and its graph)
 constexpr int VCYCLE_CLASSES = (1 << MG_K_CHEB_ZERO) | (1 << MG_K_CHEB_STEP) | (1 << MG_K_RESID) |
-                               (1 << MG_K_RESTRICT) | (1 << MG_K_PROLONG) | (1 << MG_K_BOTTOM) | (1 << MG_K_DOT);
+                               (1 << MG_K_RESTRICT) | (1 << MG_K_PROLONG) | (1 << MG_K_BOTTOM) | (1 << MG_K_DOT) |
+                               (1 << MG_K_PAIR_PRE) | (1 << MG_K_PAIR_STEP);
 
 // Runs the V-cycle (and, in mixed precision, the casts around it); through a
 // CUDA graph captured on first use when the handle enables graphs.
