@@ -787,7 +787,8 @@ template <class TV, class TC> struct Impl {
   // buffer cur (and d_{j_from-1} in Lv.d when j_from > 0), rho_prev = rho_{j_from-1}.
   // With fuse_rz the last step also accumulates rho = b.z for the outer CG and
   // finishes the CG scalars.  Returns the buffer holding the result.
-  static int cheb_steps(mg_handle* h, int l, int cur, int j_from, double rho_prev, bool fuse_rz) {
+  // d_is_x: d_{j_from-1} is the iterate itself instead (step 0 from a zero guess).
+  static int cheb_steps(mg_handle* h, int l, int cur, int j_from, double rho_prev, bool fuse_rz, bool d_is_x = false) {
     LevelBuf& Lv = h->lv[l];
     const mg_params& p = h->prm;
     double theta, delta, sigma;
@@ -804,7 +805,7 @@ template <class TV, class TC> struct Impl {
       const bool dot = fuse_rz && j + 1 == p.cheby_degree;
       TV* xo = V(Lv.x[cur ^ 1]);
       TV* dout = j + 1 < p.cheby_degree ? V(Lv.d) : nullptr;
-      const TV* dprev = j > 0 ? V(Lv.d) : nullptr;
+      const TV* dprev = j == 0 ? nullptr : d_is_x && j == j_from ? V(Lv.x[cur]) : V(Lv.d);
       int nb = -1;
       if (Lv.tma) {
         const CUtensorMap& f0 = Lv.m_full_x[cur];
@@ -847,9 +848,9 @@ template <class TV, class TC> struct Impl {
     }
     if constexpr (std::is_same<TV, double>::value) {
       if (!Lv.tma) {  // store step 0, then step 1 as an ordinary step (OpChebStart)
-        OpChebStart<TV, TV> op{V(Lv.b), V(Lv.dinv), V(Lv.x[cur]), V(Lv.d), inv_theta};
+        OpChebStart<TV, TV> op{V(Lv.b), V(Lv.dinv), V(Lv.x[cur]), nullptr, inv_theta};
         zmarch<false>(h, Lv.g, op, MG_K_CHEB_ZERO, l);
-        return cheb_steps(h, l, cur, 1, 1.0 / sigma, fuse_rz);
+        return cheb_steps(h, l, cur, 1, 1.0 / sigma, fuse_rz, true);
       }
     }
     const double rho_prev = 1.0 / sigma;

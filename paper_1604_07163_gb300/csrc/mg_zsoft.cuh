@@ -84,19 +84,31 @@ struct ZsStepP {
 __device__ __forceinline__ void zs_step_load(const OpStep64& o, int p, ZsStepP& q) {
   q.b = __ldg(o.b + p);
   q.di = __ldg(o.dinv + p);
-  if (o.dprev) q.d = __ldg(o.dprev + p);
+  if (o.dprev && o.dprev != o.x) q.d = __ldg(o.dprev + p);
+}
+// d_{j-1} at the point: after step 0 from a zero guess it is the iterate itself
+__device__ __forceinline__ double zs_d(const OpStep64& o, double xp, const ZsStepP& q) {
+  return o.dprev == o.x ? xp : q.d;
 }
 __device__ __forceinline__ void zs_step_prefetch(const OpStep64& o, int p) {
   pf_l2(o.b + p);
   pf_l2(o.dinv + p);
-  if (o.dprev) pf_l2(o.dprev + p);
+  if (o.dprev && o.dprev != o.x) pf_l2(o.dprev + p);
 }
+// A sweep's last step needs no direction: x + c1 d + c2 s as two multiply-adds
+// instead of a product, a multiply-add and an addition (with the direction that
+// is the iterate itself not read again, a step went from 274 to 231 us at 257^3).
 __device__ __forceinline__ double zs_step_emit(const OpStep64& o, int p, double S, double xp, const ZsStepP& q) {
   const double s = fma(q.di, q.b + S, -xp);
-  const double dn = o.dprev ? fma(o.c1, q.d, o.c2 * s) : s * o.inv_theta;
-  const double xn = xp + dn;
+  double xn;
+  if (o.dout) {
+    const double dn = o.dprev ? fma(o.c1, zs_d(o, xp, q), o.c2 * s) : s * o.inv_theta;
+    xn = xp + dn;
+    o.dout[p] = dn;
+  } else {
+    xn = o.dprev ? fma(o.c2, s, fma(o.c1, zs_d(o, xp, q), xp)) : fma(s, o.inv_theta, xp);
+  }
   o.xout[p] = xn;
-  if (o.dout) o.dout[p] = dn;
   return xn;
 }
 template <> struct Zs<OpStep64> : ZsBase<OpStep64, false> {
@@ -139,8 +151,8 @@ __device__ __noinline__ double zs_exact(const TU* u, const double* kx, const dou
 // What bounds it: issue slots and the float64 pipe, about evenly, over 48 bytes
 // per point of traffic.  With four float64 operations per point left on that
 // pipe the CG operator takes 166 us at 257^3 (eight: 248 us; 118 us of traffic)
-// and 1.21 ms at 513^3 (1.85 ms).  The float64 form's smoothing step keeps seven
-// (274 us, before 346 us), its residual four (168 us, before 244 us).  Measured on the
+// and 1.21 ms at 513^3 (1.85 ms).  The float64 form's smoothing step keeps six
+// (231 us a step, in float64 arithmetic 346 us), its residual four (168 us, before 244 us).  Measured on the
 // operator at 257^3: two points per thread, at 120 registers, 14 us slower; a
 // plane's loads kept in registers one plane ahead 10 to 25 us slower; 9 to 12
 // resident blocks 4 to 50 us slower.
