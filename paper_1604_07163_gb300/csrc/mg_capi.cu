@@ -122,7 +122,9 @@ struct mg_handle {
   std::vector<double> hist;
   std::string err;
   mg_stats st{};
-  std::vector<void*> allocs;
+  std::vector<void*> allocs;  // device memory, freed with the handle
+  char* chunk = nullptr;      // the chunk that alloc() hands out pieces of
+  size_t chunk_left = 0, chunk_next = 0;
   cudaGraphExec_t vexec = nullptr;
   int vexec_zcur = 0;
   bool rz_fused = false;         // last V-cycle fused rho = b.z (OpChebStepDot) into its final step
@@ -296,18 +298,45 @@ int lin_blocks(const mg_handle* h, i64 n) {
 template <class... KArgs, class... Args>
 void launch(const mg_handle* h, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, Args&&... args);
 
+// Zeroed device memory that lives as long as the handle.  A hierarchy has about
+// a hundred arrays, most of them small: they are pieces of chunks of 2 to 64 MB,
+// each allocated and zeroed at once.  Building and freeing a 129^3 hierarchy took
+// 1.9 + 1.4 ms with an allocation per array, 1.45 + 0.76 ms with chunks, of an inverse
+// problem's step of 11.4 and 10.4 ms.
+constexpr size_t ALLOC_ALIGN = 512, CHUNK_MIN = size_t(2) << 20, CHUNK_MAX = size_t(64) << 20;
+mg_status alloc_bytes(mg_handle* h, void** p, size_t bytes) {
+  bytes = (bytes + ALLOC_ALIGN - 1) / ALLOC_ALIGN * ALLOC_ALIGN;
+  if (bytes > h->chunk_left) {
+    const size_t next = h->chunk_next ? h->chunk_next : CHUNK_MIN;
+    const bool own = bytes > next / 2 && bytes > CHUNK_MIN;  // a large array: no chunk around it
+    const size_t size = own ? bytes : next;
+    void* q = nullptr;
+    cudaError_t e = cudaMalloc(&q, size);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      return fail(h, MG_ERR_ALLOC, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+    }
+    h->allocs.push_back(q);
+    e = cudaMemsetAsync(q, 0, size, h->s);
+    if (e != cudaSuccess) return fail(h, MG_ERR_CUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
+    h->chunk_next = std::min(2 * next, CHUNK_MAX);
+    if (own) {
+      *p = q;
+      return MG_OK;
+    }
+    h->chunk = (char*)q;
+    h->chunk_left = size;
+  }
+  *p = h->chunk;
+  h->chunk += bytes;
+  h->chunk_left -= bytes;
+  return MG_OK;
+}
 template <class T> mg_status alloc(mg_handle* h, T** p, i64 n) {
   void* q = nullptr;
-  cudaError_t e = cudaMalloc(&q, (size_t)n * sizeof(T));
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return fail(h, MG_ERR_ALLOC, std::string("cudaMalloc: ") + cudaGetErrorString(e));
-  }
-  h->allocs.push_back(q);
-  e = cudaMemsetAsync(q, 0, (size_t)n * sizeof(T), h->s);
-  if (e != cudaSuccess) return fail(h, MG_ERR_CUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
-  *p = (T*)q;
-  return MG_OK;
+  const mg_status s = alloc_bytes(h, &q, (size_t)n * sizeof(T));
+  if (s == MG_OK) *p = (T*)q;
+  return s;
 }
 #define AL(ptr, T, n)                                  \
   do {                                                 \
