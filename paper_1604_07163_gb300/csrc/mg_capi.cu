@@ -308,10 +308,16 @@ mg_status alloc_bytes(mg_handle* h, void** p, size_t bytes) {
   bytes = (bytes + ALLOC_ALIGN - 1) / ALLOC_ALIGN * ALLOC_ALIGN;
   if (bytes > h->chunk_left) {
     const size_t next = h->chunk_next ? h->chunk_next : CHUNK_MIN;
-    const bool own = bytes > next / 2 && bytes > CHUNK_MIN;  // a large array: no chunk around it
-    const size_t size = own ? bytes : next;
+    bool own = bytes > next / 2 && bytes > CHUNK_MIN;  // a large array: no chunk around it
+    size_t size = own ? bytes : next;
     void* q = nullptr;
     cudaError_t e = cudaMalloc(&q, size);
+    if (e != cudaSuccess && !own) {  // no room for a chunk: the array alone
+      cudaGetLastError();
+      own = true;
+      size = bytes;
+      e = cudaMalloc(&q, size);
+    }
     if (e != cudaSuccess) {
       cudaGetLastError();
       return fail(h, MG_ERR_ALLOC, std::string("cudaMalloc: ") + cudaGetErrorString(e));
