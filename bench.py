@@ -590,16 +590,13 @@ VARIANTS = {
 # the kernel and traffic is reported as null.
 NCU_TRAFFIC = {
     # (workload, form, class): (DRAM bytes per launch, CUDA-source hash at capture)
-    # cheb_step: mean of the two finest-level launches per V-cycle (step 0:
-    # 450.1 MB; step 1 with b.z: 460.8 MB)
-    ("poisson257_c1e4", "mixed_fp32", "cheb_step"): (455.5e6, "f8447c71119a0be7"),
-    ("poisson257_c1e4", "mixed_fp32", "cheb_zero"): (396.5e6, "f8447c71119a0be7"),
-    ("poisson257_c1e4", "mixed_fp32", "resid"): (392.4e6, "f8447c71119a0be7"),
-    ("poisson257_c1e4", "mixed_fp32", "prolong"): (79.0e6, "f8447c71119a0be7"),
-    ("poisson257_c1e4", "mixed_fp32", "restrict"): (66.9e6, "f8447c71119a0be7"),
-    ("poisson257_c1e4", "mixed_fp32", "cg_apply"): (788.8e6, "f8447c71119a0be7"),
-    ("poisson257_c1e4", "mixed_fp32", "cg_dir"): (547.4e6, "f8447c71119a0be7"),
-    ("poisson257_c1e4", "mixed_fp32", "cg_upd"): (413.4e6, "f8447c71119a0be7"),
+    ("poisson257_c1e4", "mixed_fp32", "pair_step"): (474.9e6, "0dae3af666c83302"),
+    ("poisson257_c1e4", "mixed_fp32", "pair_pre"): (467.2e6, "0dae3af666c83302"),
+    ("poisson257_c1e4", "mixed_fp32", "prolong"): (78.8e6, "0dae3af666c83302"),
+    ("poisson257_c1e4", "mixed_fp32", "restrict"): (66.8e6, "0dae3af666c83302"),
+    ("poisson257_c1e4", "mixed_fp32", "cg_apply"): (790.6e6, "0dae3af666c83302"),
+    ("poisson257_c1e4", "mixed_fp32", "cg_dir"): (547.5e6, "0dae3af666c83302"),
+    ("poisson257_c1e4", "mixed_fp32", "cg_upd"): (413.7e6, "0dae3af666c83302"),
 }
 
 

@@ -1,5 +1,5 @@
-"""The vector kernels of the transfers and of the 27-point passes give the
-one-point-per-thread kernels' results bit for bit: rows that end inside a
+"""The vector kernels of the transfers, of the float32 7-point passes and of the
+27-point passes give the one-point-per-thread kernels' results bit for bit: rows that end inside a
 vector, rows wider than a warp's, level sizes down to three points."""
 import numpy as np
 import pytest
@@ -35,6 +35,17 @@ def test_transfers(gpu_lib, dims, precision):
         # the restriction alone: with x = 0 the residual is b in either kernel
         z = torch.zeros_like(x)
         assert torch.equal(A.residual_restrict(b, z, l), B.residual_restrict(b, z, l))
+
+
+@pytest.mark.parametrize("dims", DIMS)
+@pytest.mark.parametrize("precision", ["mixed_fp32", "mixed_bf16k"])
+@pytest.mark.parametrize("degree", [2, 3])
+def test_7_point_smoothing(gpu_lib, dims, precision, degree):
+    A, B = pair(gpu_lib, dims, precision=precision, cheby_degree=degree)
+    for l in range(A.num_levels):
+        b, x = (T(mi.random_nodal(A.level_shape(l), 66 + i)) for i in range(2))
+        assert torch.equal(A.smooth(b, None, l), B.smooth(b, None, l))
+        assert torch.equal(A.smooth(b, x, l), B.smooth(b, x, l))
 
 
 @pytest.mark.parametrize("dims", DIMS)
