@@ -2864,7 +2864,8 @@ mg_status mg_gradient(mg_handle* h, const double* phi, const double* lambda, dou
   const bool am = h->prm.face_rule != 0;
   const double w[3] = {am ? L0.ih2[0] : 1.0 / L0.ih2[0], am ? L0.ih2[1] : 1.0 / L0.ih2[1],
                        am ? L0.ih2[2] : 1.0 / L0.ih2[2]};
-  k_gradient<<<grid, DN_THREADS, 0, h->s>>>(L0.kc, phi, lambda, L0.kx64, L0.ky64, L0.kz64, g, w[0], w[1], w[2],
+  const int lg = std::ilogb(std::max(L0.ih2[0], std::max(L0.ih2[1], L0.ih2[2])));
+  k_gradient<<<grid, DN_THREADS, 0, h->s>>>(L0.kc, phi, lambda, L0.kx64, L0.ky64, L0.kz64, g, w[0], w[1], w[2], lg,
                                             h->prm.face_rule, kc, grad);
   CKL();
   return MG_OK;

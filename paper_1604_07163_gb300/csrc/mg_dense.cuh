@@ -117,17 +117,20 @@ __global__ void __launch_bounds__(DN_THREADS, 8)
 // -(dlam dphi K_e^2) h_a^2 / (4 k_c): the 12 means (5 float64 divisions each)
 // need not be formed again, and an edge's value does not depend on the cell.
 // wx, wy, wz are h_a^2 (harmonic) or h_a^-2 (arithmetic).
+// K_e^2 may leave the range where k^2 / k does not, so a warp takes a power of
+// two out of its K_e, near the reciprocal of its first cell's k 2^lg (2^lg about
+// the largest h_a^-2), and puts it back at the end: neither changes a bit.
 //
 // What bounds it: the float64 pipe, about 43 operations per cell (one
 // division among them); the 60 divisions per cell of the twelve means took
-// 2.28 ms at 129^3, this kernel takes 0.29 ms with its call.  A thread owns the nodes (I, J) and (I, J + 1) of a
+// 2.28 ms at 129^3, this kernel takes 0.25 ms with its call.  A thread owns the nodes (I, J) and (I, J + 1) of a
 // column and walks node planes; the edges of column I + 1 come from the next
 // lane (31 cells per warp), those of the plane below stay in registers.
 constexpr int GR_TX = 31;
 __global__ void __launch_bounds__(DN_THREADS)
     k_gradient(const double* __restrict__ kc, const double* __restrict__ phi, const double* __restrict__ lam,
                const double* __restrict__ kx, const double* __restrict__ ky, const double* __restrict__ kz, Geom g,
-               double wx, double wy, double wz, int face_rule, int kchunk, double* __restrict__ grad) {
+               double wx, double wy, double wz, int lg, int face_rule, int kchunk, double* __restrict__ grad) {
   const int lane = threadIdx.x & 31;
   const int cx = g.nx + 1, cy = g.ny + 1, cz = g.nz + 1;  // cells
   const int I = min(blockIdx.x * GR_TX + lane, cx), J = blockIdx.y * DN_TY + (threadIdx.x >> 5);
@@ -140,10 +143,18 @@ __global__ void __launch_bounds__(DN_THREADS)
   i64 q = (i64)K0 * sz + (i64)J * sy + I;
   int p = (int)g.at(I - 1, J - 1, K0 - 1);
   double lm0 = 0.0, lm1 = 0.0, pm0 = 0.0, pm1 = 0.0, Pm = 0.0;
+  // x: the exponent of the warp's first cell's k 2^lg; 2^x and 4 2^-x
+  const unsigned long long first = dbits(__ldg(kc + ((i64)K0 * cy + J) * cx + blockIdx.x * GR_TX));
+  const int x = min(max((int)(first >> 52) - 1023 + lg, -1000), 1000), dx = x * (1 << 20);
+  const double up = bitsd((unsigned long long)(1023 + x) << 52), down4 = bitsd((unsigned long long)(1025 - x) << 52);
   auto edge = [&](double dl, double dp, const double* k, int at) {
     const double t = dl * dp;
     if (face_rule) return t;
-    const double c = __ldg(k + at);
+    // 2^-x K by its exponent bits (five float64 products per cell more took 277 us instead of 247 at
+    // 129^3).  A zero (t is 0 there) or a value out of range becomes some finite number.
+    const double K = __ldg(k + at);
+    const int hi = min(max(__double2hiint(K) - dx, 0), 0x7fe00000);
+    const double c = __hiloint2double(hi, __double2loint(K));
     return t * (c * c);
   };
   auto east = [](double v) { return __shfl_down_sync(0xffffffffu, v, 1); };
@@ -161,7 +172,7 @@ __global__ void __launch_bounds__(DN_THREADS)
       if (out) {
         const i64 c = ((i64)(K - 1) * cy + J) * cx + I;
         const double k = __ldg(kc + c);
-        grad[c] = face_rule ? -0.25 * k * acc : -acc / (4.0 * k);
+        grad[c] = face_rule ? -0.25 * k * acc : up * (-acc / (down4 * k));
       }
     }
     lm0 = l0, lm1 = l1, pm0 = p0, pm1 = p1, Pm = P;

@@ -32,3 +32,19 @@ def test_restriction_of_large_residuals(gpu_lib, dims, precision):
         assert torch.equal(got, B.residual_restrict(b, z, l))
     A.close()
     B.close()
+
+
+@pytest.mark.parametrize("dims", [(9, 17, 33), (41, 49, 129)])
+@pytest.mark.parametrize("face_rule", [0, 1])
+@pytest.mark.parametrize("ek,ex", [(500, 0), (400, 160), (-500, -60)])
+def test_cell_gradient_scales_with_its_operands(gpu_lib, dims, face_rule, ek, ex):
+    """k times 2^ek, phi and lambda times 2^ex: the gradient times 2^(ek + 2 ex), bit for bit (h^-4 k^2 and its products
+    with dphi dlambda would leave the range, h^-2 k and the gradient do not)."""
+    mg = gpu_lib
+    k, x, lam = (mi.cell_k(dims, 2, -1.0, 1.0, 91), mi.random_nodal(dims, 92), mi.random_nodal(dims, 93))
+    g = []
+    for a, b in ((0, 0), (ek, ex)):
+        S = mg.MGSolver(T(np.ldexp(k, a)), mg.Params(face_rule=face_rule))
+        g.append(S.gradient(T(np.ldexp(x, b)), T(np.ldexp(lam, b))).cpu().numpy())
+        S.close()
+    assert np.array_equal(g[1], np.ldexp(g[0], ek + 2 * ex))
