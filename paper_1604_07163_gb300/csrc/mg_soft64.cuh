@@ -117,4 +117,11 @@ __host__ __device__ __forceinline__ bool soft_sum4(const S64 (&u)[4], const S64 
   return (unsigned)(M - 1340) < 1480u && top != 0;
 }
 
+// Whether all four are zeros; their sum in z (-0 where all are -0).
+__device__ __forceinline__ bool all_zero(double a, double b, double c, double d, double& z) {
+  const unsigned long long some = dbits(a) | dbits(b) | dbits(c) | dbits(d);
+  z = bitsd(dbits(a) & dbits(b) & dbits(c) & dbits(d));
+  return some << 1 == 0;
+}
+
 }  // namespace mgdev
