@@ -1387,14 +1387,6 @@ mg_status unpack_level(mg_handle* h, int l, const void* src, double* dst, bool f
 
 bool overlap(const double* a, i64 na, const double* b, i64 nb) { return a < b + nb && b < a + na; }
 
-// The two dense device nodal arrays of mg_solve_host, on first use.
-mg_status host_stage(mg_handle* h) {
-  if (h->hstage[1]) return MG_OK;
-  const LevelBuf& L0 = h->lv[0];
-  for (double*& b : h->hstage) AL(b, double, (i64)L0.N[0] * L0.N[1] * L0.N[2]);
-  return MG_OK;
-}
-
 // Galerkin level l: A_l = R A_{l-1} P in float64 from the level above (its
 // 7-point edge coefficients or its 27-point couplings), then the V-cycle
 // precision copies, D^-1 and the Gershgorin bound of D^-1 A_l.
@@ -2822,8 +2814,9 @@ mg_status mg_solve_host(mg_handle* h, const double* f_host, double* x_host, doub
   const LevelBuf& L0 = h->lv[0];
   const size_t bytes = sizeof(double) * (size_t)L0.N[0] * L0.N[1] * L0.N[2];
   Guard guard(h);
-  mg_status s = host_stage(h);
-  if (s != MG_OK) return s;
+  if (!h->hstage[1])
+    for (double*& b : h->hstage) AL(b, double, (i64)(bytes / sizeof(double)));
+  mg_status s;
   CK(cudaMemcpyAsync(h->hstage[0], f_host, bytes, cudaMemcpyHostToDevice, h->s));
   if (h->prm.nonzero_guess) CK(cudaMemcpyAsync(h->hstage[1], x_host, bytes, cudaMemcpyHostToDevice, h->s));
   if (h->nslab > 1)
@@ -2847,16 +2840,10 @@ mg_status mg_gradient(mg_handle* h, const double* phi, const double* lambda, dou
   Guard guard(h);
   const LevelBuf& L0 = h->lv[0];
   const Geom& g = L0.g;
-  // a gradient array that overlaps an input is formed from a copy of it
+  // a gradient array that overlaps an input is formed in a CG vector (whose pads are zero between calls) and copied
   const i64 nodes = (i64)L0.N[0] * L0.N[1] * L0.N[2], cells = (i64)(L0.N[0] - 1) * (L0.N[1] - 1) * (L0.N[2] - 1);
-  const double** in[2] = {&phi, &lambda};
-  for (int a = 0; a < 2; ++a)
-    if (overlap(*in[a], nodes, grad, cells)) {
-      mg_status s = host_stage(h);
-      if (s != MG_OK) return s;
-      CK(cudaMemcpyAsync(h->hstage[a], *in[a], sizeof(double) * nodes, cudaMemcpyDeviceToDevice, h->s));
-      *in[a] = h->hstage[a];
-    }
+  const bool staged = overlap(phi, nodes, grad, cells) || overlap(lambda, nodes, grad, cells);
+  double* out = staged ? h->cq : grad;
   dim3 grid((g.nx + 1 + GR_TX - 1) / GR_TX, (g.ny + 1 + DN_TY - 1) / DN_TY, 1);
   const int zs = best_zsplit(grid.x * grid.y, h->nsm * 6, g.nz + 1, 4);
   const int kc = (g.nz + 1 + zs - 1) / zs;
@@ -2866,8 +2853,12 @@ mg_status mg_gradient(mg_handle* h, const double* phi, const double* lambda, dou
                        am ? L0.ih2[2] : 1.0 / L0.ih2[2]};
   const int lg = std::ilogb(std::max(L0.ih2[0], std::max(L0.ih2[1], L0.ih2[2])));
   k_gradient<<<grid, DN_THREADS, 0, h->s>>>(L0.kc, phi, lambda, L0.kx64, L0.ky64, L0.kz64, g, w[0], w[1], w[2], lg,
-                                            h->prm.face_rule, kc, grad);
+                                            h->prm.face_rule, kc, out);
   CKL();
+  if (staged) {
+    CK(cudaMemcpyAsync(grad, out, sizeof(double) * cells, cudaMemcpyDeviceToDevice, h->s));
+    CK(cudaMemsetAsync(out, 0, sizeof(double) * cells, h->s));
+  }
   return MG_OK;
 }
 
