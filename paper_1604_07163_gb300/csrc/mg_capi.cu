@@ -98,7 +98,6 @@ struct mg_handle {
   int bot_cluster = 1;  // blocks of the bottom kernel (a cluster when > 1)
   int bot_smem = 0;     // blocks of the bottom kernel in shared memory (0: it does not fit, k_bottom runs)
   LevelBuf lv[MG_MAX_LEVELS];
-  double* Lc = nullptr;  // Cholesky factor of the coarsest operator
   double* Ai = nullptr;  // inverse of the coarsest operator
   double* Ac = nullptr;  // the dense coarsest operator (inexact coarse solve)
   // flexible GMRES: basis V_0..V_m (float64), preconditioned Z_0..Z_{m-1}
@@ -1730,30 +1729,35 @@ mg_status build_hierarchy(mg_handle* h, int Nx, int Ny, int Nz, const double* k,
         }))
       h->bot_smem = nb;
   }
-  // coarsest operator: dense float64 assembly and Cholesky factorisation
-  AL(h->Lc, double, (i64)h->nc * h->nc);
+  // coarsest operator: dense float64 assembly, Cholesky factorisation, inverse (which takes the factor's place)
+  const i64 nn = (i64)h->nc * h->nc;
+  double *X = nullptr, *rows = nullptr;
+  AL(h->Ai, double, nn);
+  AL(X, double, nn);
+  AL(rows, double, 27 * (i64)h->nc);
   const LevelBuf& Cv = h->lv[L - 1];
-  if (Cv.g27) k_assemble_dense27<<<lin_blocks(h, h->nc), 256, 0, h->s>>>(Cv.w64, Cv.dg64, Cv.g, h->Lc);
-  else k_assemble_dense<<<lin_blocks(h, h->nc), 256, 0, h->s>>>(Cv.kx64, Cv.ky64, Cv.kz64, Cv.g, h->Lc);
+  if (Cv.g27) k_assemble_dense27<<<lin_blocks(h, h->nc), 256, 0, h->s>>>(Cv.w64, Cv.dg64, Cv.g, h->Ai);
+  else k_assemble_dense<<<lin_blocks(h, h->nc), 256, 0, h->s>>>(Cv.kx64, Cv.ky64, Cv.kz64, Cv.g, h->Ai);
   CKL();
   if (p.coarse_solve == 1) {  // keep the operator for the inexact solve
     if (h->nc > 32) return fail(h, MG_ERR_ARG, "the inexact coarse solve needs at most 32 coarsest unknowns");
-    AL(h->Ac, double, (i64)h->nc * h->nc);
-    CK(cudaMemcpyAsync(h->Ac, h->Lc, sizeof(double) * h->nc * h->nc, cudaMemcpyDeviceToDevice, h->s));
+    AL(h->Ac, double, nn);
+    CK(cudaMemcpyAsync(h->Ac, h->Ai, sizeof(double) * nn, cudaMemcpyDeviceToDevice, h->s));
   }
   if (p.test_inject == 2) {  // test only: a coarsest operator that is not positive definite
-    k_scale_strided<<<1, 256, 0, h->s>>>(h->Lc, -1.0, (i64)h->nc, (i64)h->nc + 1);
+    k_scale_strided<<<1, 256, 0, h->s>>>(h->Ai, -1.0, (i64)h->nc, (i64)h->nc + 1);
     CKL();
   }
+  k_coarse_rows<<<lin_blocks(h, 27 * (i64)h->nc), 256, 0, h->s>>>(h->Ai, rows, Cv.g);
   CK(cudaMemsetAsync(h->dflag, 0, sizeof(int), h->s));
-  k_cholesky<<<1, 1024, 0, h->s>>>(h->Lc, h->nc, h->dflag);
+  k_cholesky<<<1, 1024, 0, h->s>>>(h->Ai, h->nc, h->dflag);
   CKL();
   int bad = 0;
   CK(cudaMemcpyAsync(&bad, h->dflag, sizeof(int), cudaMemcpyDeviceToHost, h->s));
   CK(cudaStreamSynchronize(h->s));
   if (bad) return fail(h, MG_ERR_NOT_SPD, "coarsest operator is not positive definite");
-  AL(h->Ai, double, (i64)h->nc * h->nc);
-  k_coarse_inverse<<<(h->nc + 3) / 4, 128, 0, h->s>>>(h->Lc, h->Ai, h->nc);
+  k_coarse_inverse<<<(h->nc + 3) / 4, 128, 0, h->s>>>(h->Ai, X, h->nc);
+  k_coarse_refine<<<(h->nc + 3) / 4, 128, 0, h->s>>>(rows, X, h->Ai, Cv.g, h->nc);
   CKL();
   return MG_OK;
 }
