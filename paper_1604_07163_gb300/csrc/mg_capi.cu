@@ -1733,7 +1733,23 @@ mg_status build_hierarchy(mg_handle* h, int Nx, int Ny, int Nz, const double* k,
   const i64 nn = (i64)h->nc * h->nc;
   double *X = nullptr, *rows = nullptr;
   AL(h->Ai, double, nn);
-  AL(X, double, nn);
+  // Setup's copy of the inverse: up to 1 MB (362 unknowns) a piece of a chunk; a larger one, up to 8 MB, is given back
+  struct Scratch {
+    cudaStream_t s;
+    void* p = nullptr;
+    ~Scratch() {
+      if (p && cudaStreamSynchronize(s) == cudaSuccess) cudaFree(p);
+    }
+  } scratch{h->s};
+  if (nn * (i64)sizeof(double) <= 1 << 20) {
+    AL(X, double, nn);
+  } else {
+    if (cudaMalloc(&scratch.p, nn * sizeof(double)) != cudaSuccess) {
+      cudaGetLastError();
+      return fail(h, MG_ERR_ALLOC, "cudaMalloc: out of memory");
+    }
+    X = (double*)scratch.p;
+  }
   AL(rows, double, 27 * (i64)h->nc);
   const LevelBuf& Cv = h->lv[L - 1];
   if (Cv.g27) k_assemble_dense27<<<lin_blocks(h, h->nc), 256, 0, h->s>>>(Cv.w64, Cv.dg64, Cv.g, h->Ai);
