@@ -465,7 +465,7 @@ dim3 zs_grid(const mg_handle* h, const Geom& g, int* kchunk) {
 
 // Launch geometry of the vector drivers, np points per thread: 2^lw lanes per
 // row, the smallest power of two up to a warp that covers it, and plane chunks
-// by wave efficiency over `blocks` resident blocks per SM, of at least `least`
+// by wave efficiency over `blocks` blocks per SM, of at least `least`
 // planes where that leaves two waves of blocks (k_zvec reads two planes more
 // than it writes: at 257^3 chunks of 3 planes took 121 us a step, of 9 82 us).
 dim3 vec_grid(const mg_handle* h, const Geom& g, int np, int blocks, int least, int* lw, int* kchunk) {
@@ -605,7 +605,7 @@ int zmarch(mg_handle* h, const Geom& g, const Op& op, int cls = -1, int level = 
   if constexpr (Zv<Op>::ok) {
     if (h->zvec) {
       int lw;
-      dim3 grid = vec_grid(h, g, Zv<Op>::NP, ZV_BLOCKS, ZV_CHUNK, &lw, &kc);
+      dim3 grid = vec_grid(h, g, Zv<Op>::NP, zv_share(Zv<Op>::NP), zv_chunk(Zv<Op>::NP), &lw, &kc);
       const int e = cls >= 0 ? tm_begin(h, cls, level) : -1;
       launch(h, k_zvec<Op, RED>, grid, dim3(ZV_THREADS), 0, op, g, lw, kc, h->partials, h->pstride);
       ++h->launches;
@@ -1691,7 +1691,7 @@ mg_status build_hierarchy(mg_handle* h, int Nx, int Ny, int Nz, const double* k,
   {
     int lwz;
     for (int np : {2, 4}) {
-      dim3 gv = vec_grid(h, h->lv[0].g, np, ZV_BLOCKS, ZV_CHUNK, &lwz, &kcz);
+      dim3 gv = vec_grid(h, h->lv[0].g, np, zv_share(np), zv_chunk(np), &lwz, &kcz);
       const int vg = gv.x * gv.y * gv.z;
       if (h->pstride < vg) h->pstride = vg;
     }
@@ -2167,7 +2167,7 @@ mg_status build_slabs(mg_handle* h) {
     c->pstride = std::max(std::max((int)(gz.x * gz.y * gz.z), (int)(gs.x * gs.y * gs.z)), c->lin_grid);
     int lwz;
     for (int np : {2, 4}) {
-      dim3 gv = vec_grid(c, g0, np, ZV_BLOCKS, ZV_CHUNK, &lwz, &kcz);
+      dim3 gv = vec_grid(c, g0, np, zv_share(np), zv_chunk(np), &lwz, &kcz);
       c->pstride = std::max(c->pstride, (int)(gv.x * gv.y * gv.z));
     }
     {

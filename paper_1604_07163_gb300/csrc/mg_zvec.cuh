@@ -183,17 +183,35 @@ template <class R, class TV, class TC, int NP>
 __device__ __forceinline__ void zv_step_emit(const OpChebStep<R, TV, TC>& o, int p, int nv, const ZvNb<R, NP>& nb,
                                              const ZvStepP<R, TV, TC>& P, R (&xn)[NP]) {
   R dn[NP];
+  if constexpr (sizeof(R) == 4) {
 #pragma unroll
-  for (int e = 0; e < NP; ++e) {
-    R D;
-    const R S = nb.eval(e, D);
-    const R xp = nb.uc[e];
-    R inv;
-    if constexpr (sizeof(R) == 4) inv = (R)1 / D;
-    else inv = P.di[e];
-    const R s = fma(inv, P.b[e] + S, -xp);
-    dn[e] = o.dprev ? fma(o.c1, P.d[e], o.c2 * s) : s * o.inv_theta;
-    xn[e] = xp + dn[e];
+    for (int e = 0; e < NP; ++e) {
+      R D;
+      const R S = nb.eval(e, D);
+      const R xp = nb.uc[e];
+      const R s = fma((R)1 / D, P.b[e] + S, -xp);
+      dn[e] = o.dprev ? fma(o.c1, P.d[e], o.c2 * s) : s * o.inv_theta;
+      xn[e] = xp + dn[e];
+    }
+  } else {
+    // one branch for all points: a selection formed both directions, on the float64 pipe (step at 257^3 390 us,
+    // this 344)
+    R s[NP];
+#pragma unroll
+    for (int e = 0; e < NP; ++e) {
+      R D;
+      const R S = nb.eval(e, D);
+      s[e] = fma(P.di[e], P.b[e] + S, -nb.uc[e]);
+    }
+    if (o.dprev) {
+#pragma unroll
+      for (int e = 0; e < NP; ++e) dn[e] = fma(o.c1, P.d[e], o.c2 * s[e]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < NP; ++e) dn[e] = s[e] * o.inv_theta;
+    }
+#pragma unroll
+    for (int e = 0; e < NP; ++e) xn[e] = __dadd_rn(nb.uc[e], dn[e]);
   }
   stn(o.xout + p, xn, nv);
   if (o.dout) stn(o.dout + p, dn, nv);
@@ -424,7 +442,13 @@ template <class TB> struct Zv<OpResidualD<TB>> {
 // zero-guess step, step and residual at 257^3 with 4, 5 and 6 blocks 81 / 84 / 68,
 // 77 / 82 / 65 and 104 / 94 / 72 us.
 constexpr int ZV_BLOCKS = 5;
-constexpr int ZV_CHUNK = 8;  // least planes per block on large levels
+// Blocks per SM that the plane chunks are cut for, and least planes per chunk on
+// large levels, by points per thread.  Two (float64) is bound by the float64 pipe
+// and wants even shares more than few planes read twice: 2 x 5 and 4 instead of 5
+// and 8 take 159 instead of 168 us a step at 193^3, 52.6 instead of 55.9 at 129^3, the
+// same at 257^3 and 321^3.
+constexpr int zv_share(int np) { return np == 2 ? 2 * ZV_BLOCKS : ZV_BLOCKS; }
+constexpr int zv_chunk(int np) { return np == 2 ? 4 : 8; }
 
 // The driver: 2^lw lanes per row (whole rows in a warp, so that every shuffle
 // stays inside a row), ZV_THREADS / 2^lw rows per block.  Lanes past the row
