@@ -56,7 +56,7 @@ def bytes_per_point(cls: str, v: int, c: int, degree: int = 2, fp64: bool = Fals
         "cheb_zero": 3 * v + c + (v if degree > 2 else 0),  # read b, dinv, k; write x (and d)
         "cheb_step": 4 * v + c + dinv,                    # (x+b+k+x'+d) and (x+d+b+k+z), averaged
         "resid": 3 * v + c,                               # read x, b, k; write r
-        "pair_pre": 4 * v + c,                            # read b, dinv (or x), k; write x, r
+        "pair_pre": (4 if degree > 1 else 5) * v + c,     # read b, dinv, k (after a step, degree 1, x too); write x, r
         "pair_step": 4 * v + c,                           # read x, b, dinv, k; write z
         "restrict": 9 * v,                                # per coarse point: read 8 fine r, write 1
         "prolong": 2 * v + v / 8,                         # read x, e/8; write x

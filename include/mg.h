@@ -8,9 +8,10 @@
  * recursively; per-level components of Sec. 2.1.1) with re-discretised coarse
  * operators (Sec. 1, Sec. 4.3), a Jacobi-preconditioned Chebyshev smoother
  * (Sec. 4.3), full-weighting restriction, trilinear prolongation, and an exact
- * dense Cholesky solve of the coarsest operator (Sec. 1, Sec. 3.3.1).  Coarse
- * levels too small to fill the GPU run on progressively fewer thread blocks and
- * finally inside one persistent thread block: the single-GPU analogue of
+ * dense solve of the coarsest operator (Sec. 1, Sec. 3.3.1): a product with its
+ * inverse, formed at setup from the Cholesky factor.  Coarse levels too small to
+ * fill the GPU run on progressively fewer thread blocks and finally inside one
+ * thread-block cluster, in its shared memory: the single-GPU analogue of
  * agglomerating a coarse problem onto fewer ranks (Sec. 3, Sec. 3.1).  The
  * outer Krylov method is CG (Sec. 2.1), stopped when the residual 2-norm falls
  * below rtol times that of b (Sec. 4.2, Sec. 4.3).
@@ -106,14 +107,16 @@ typedef struct {
                           or one thread-block cluster (bottom_blocks) (default 4096) */
   int use_graph;       /* 1: replay the V-cycle from a captured CUDA graph (default 1) */
   int stencil_kernel;  /* smoother/residual kernels on the levels above the bottom kernel:
-                          0 (default) z-marching, 64x4 tiles of two consecutive points per
-                            thread: vector loads, x neighbours by warp shuffles, z neighbours
-                            in registers, L2 prefetch two planes ahead (the fastest measured
+                          0 (default) z-marching: float32 and 27-point passes with four consecutive
+                            points per thread (vector loads, x neighbours by warp shuffles), on
+                            large 7-point levels two passes per sweep; float64 passes with part of
+                            their products on the integer pipe (two points per thread in float64
+                            arithmetic where k lies outside 2^-150 .. 2^150) (the fastest measured
                             on GB300),
                           1 TMA-staged tiles (cp.async.bulk.tensor into an mbarrier-tracked ring of
                             shared-memory stages; every wait bounded),
-                          2 z-marching with one point per thread and neighbours read through L1 (the
-                            driver the float64 CG operator and the 27-point passes always use) */
+                          2 z-marching with one point per thread and neighbours read through L1, for
+                            every pass, the float64 CG operator and the 27-point ones included */
   int use_pdl;         /* 1: launch solve kernels as programmatic dependent launches (default 1) */
   int smoother;        /* mg_smoother (default MG_SMOOTHER_CHEBYSHEV).  With Richardson, nu_pre and
                           nu_post count iterations and cheby_degree, eig_lo_frac, eig_hi are unused */
@@ -129,7 +132,7 @@ typedef struct {
                           a 10-step CG-Lanczos estimate of the largest eigenvalue of D^-1 A on the level,
                           from a seeded random right-hand side (computed at setup) */
   double eig_safety;   /* upper factor of eig_mode 1 (default 1.1) */
-  int coarse_solve;    /* coarsest solve: 0 (default) dense Cholesky; 1 GMRES preconditioned with
+  int coarse_solve;    /* coarsest solve: 0 (default) exact, by the dense inverse; 1 GMRES preconditioned with
                           Jacobi, stopped at coarse_rtol (the inexact, truncated coarse solve of Sec. 5;
                           the V-cycle is then no longer a fixed linear operator: use MG_KRYLOV_FGMRES).
                           1 needs a coarsest level of at most 32 unknowns */
@@ -193,7 +196,7 @@ mg_status mg_params_default(mg_params* p);
  * stream is a cudaStream_t (NULL = default stream).  On success *h owns all
  * device buffers of the hierarchy.  Setup follows Eq. 2 with the face rule of
  * p->face_rule on every level and the coarse rule of p->coarse_k_rule between
- * levels, and factors the coarsest operator with a dense Cholesky. */
+ * levels, factors the coarsest operator with a dense Cholesky and inverts it. */
 mg_status mg_setup(mg_handle** h, int Nx, int Ny, int Nz, const double* k_cells, int k_on_device,
                    const mg_params* p, void* stream);
 
@@ -301,7 +304,8 @@ mg_status mg_residual_restrict(mg_handle* h, int l, const double* b, const doubl
 /* x += P ec: trilinear prolongation from level l+1 to level l (Algorithm 1,
  * prolongation step). */
 mg_status mg_prolong_add(mg_handle* h, int l, const double* ec, double* x);
-/* x = A_L^-1 b on the coarsest level by the dense Cholesky factor. */
+/* x = A_L^-1 b on the coarsest level: a product with the dense inverse, whose entries are correct to
+ * one float64 rounding (or the inexact solve, coarse_solve 1). */
 mg_status mg_coarse_solve(mg_handle* h, const double* b, double* x);
 /* z = M^-1 r: one V-cycle with zero initial guess from the finest level. */
 mg_status mg_vcycle(mg_handle* h, const double* r, double* z);
@@ -374,17 +378,17 @@ mg_status mg_timing_enable(mg_handle* h, int class_mask, int level_mask);
 mg_status mg_timing_read(const mg_handle* h, int cls, int l, double* ms, long long* launches, double* points);
 
 /* ---- float64 FMA throughput (measurement helper; not part of the method) --
- * The outer Krylov operator q = A p in float64 does eight float64 FMAs per
- * finest point against one neighbour load each, so on GPUs with a narrow
- * float64 pipe its bound is the float64 FMA rate, not memory bandwidth.  This
- * call times a kernel of independent FMA chains on the current device (8 per
+ * The float64 stencils do 8 to 11 float64 operations per point, so on GPUs with
+ * a narrow float64 pipe their bound in float64 arithmetic is its rate, not memory
+ * bandwidth (the reason why the default kernels form part of the products on
+ * the integer pipe).  This call times a kernel of independent FMA chains on the current device (8 per
  * thread, 4 blocks of 256 threads per SM, about 16 ms per launch on a GPU with
  * two float64 FMAs per clock per SM) on a stream of its own, one untimed launch
  * and then `launches` (1..100) launches timed with CUDA events, and writes the
  * fastest launch's rate to *tflops in TFLOP/s (one FMA = 2 flops).  The figure
  * is a lower bound on the float64 pipe's rate, not its peak: on GB300 it reads
  * about 0.84 of the nominal two FMAs per clock per SM, and long launches of the
- * float64 operator run faster than it.
+ * float64 operator in float64 arithmetic run faster than it.
  * Allocates and frees a small device buffer; synchronises its own stream.
  * Returns MG_ERR_ARG for launches outside 1..100 or a null tflops, MG_ERR_CUDA
  * if a CUDA call fails. */

@@ -23,7 +23,7 @@
 //
 // Measured for the levels 15^3, 7^3, 3^3 (one launch timed alone, launch
 // included): float32 28 -> 21 us, float64 56 -> 33 us, 27-point bfloat16
-// couplings 39 -> 23 us; the whole 33^3 float64 solve 1.42 -> 1.05 ms.  Eight
+// couplings 39 -> 23 us; the whole 33^3 float64 solve 1.5 -> 1.1 ms.  Eight
 // blocks are the fastest throughout (float64 89 / 70 / 42 / 33 us for 1 (in
 // k_bottom) / 2 / 4 / 8; float32 28 / 27 / 23 / 21).  A cluster barrier
 // with remote stores before it takes 830 to 900 cycles, a pass of a 7^3 level

@@ -7,9 +7,10 @@
 // of planes of a (4 * 2^lx) x (PR_THREADS / 2^lx) tile: the first pass is formed
 // on the whole tile, its plane goes to the neighbours through shared memory,
 // and the second pass follows one plane behind on the tile's interior.  The
-// coefficients, the right-hand side and 1 / D are read once and the
-// intermediate iterate and direction never leave the SM: 28 bytes per
-// point instead of 48 to 56.  The price is the first pass on the tile's rim
+// coefficients, the right-hand side and 1 / D are read once, the direction never
+// leaves the SM and the iterate between the passes only where the residual form
+// stores it: 28 bytes per point (a step and the residual 32) instead of 48 to
+// 56.  The price is the first pass on the tile's rim
 // (one row on either side, one plane on either side of a chunk, and four points
 // on either side where a row is wider than the tile).
 //

@@ -1,8 +1,8 @@
-// Float64 FMA throughput of the current device, the unit that bounds the
-// outer Krylov operator (eight float64 FMAs per finest point, one neighbour
-// load each) on GPUs whose float64 pipe is narrow.  A measurement helper for
-// roofline figures; no solve calls it.  What it times is a lower bound on the
-// pipe's rate: on GB300 long launches of the float64 operator run faster.
+// Float64 FMA throughput of the current device, the unit that bounds the float64
+// stencils in float64 arithmetic (8 to 11 operations per point) on GPUs whose
+// float64 pipe is narrow.  A measurement helper for callers' roofline figures; no
+// solve calls it.  What it times is a lower bound on the pipe's rate: on GB300 long
+// launches of the one-point-per-thread float64 operator run faster.
 //
 // Every thread runs PK_CHAINS independent recurrences a <- a * m + c, so the
 // float64 pipe has independent instructions to issue.  With m = 1 - 2^-10 and
