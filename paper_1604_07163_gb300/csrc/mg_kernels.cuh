@@ -354,14 +354,21 @@ __global__ void __launch_bounds__(128) k_coarse_refine(const double* __restrict_
   const double* x = X + (i64)c * n;
   for (int q = lane; q < n; q += 32) {
     double s = q == c ? 1.0 : 0.0, e = 0.0;
-    for (int o = 0; o < 27; ++o) {
-      const double a = __ldg(B + (i64)o * n + q);
-      if (a == 0.0) continue;
-      const double xv = __ldg(x + q + ((o / 9 - 1) * g.ny + o / 3 % 3 - 1) * g.nx + o % 3 - 1);
-      const double p = __dmul_rn(-a, xv), pe = fma(-a, xv, -p);
-      const double t = __dadd_rn(s, p), w = __dsub_rn(t, s);
-      e = __dadd_rn(e, __dadd_rn(__dadd_rn(__dsub_rn(s, __dsub_rn(t, w)), __dsub_rn(p, w)), pe));
-      s = t;
+    for (int z = 0; z < 3; ++z) {
+      double a[9], xv[9];
+#pragma unroll
+      for (int o = 0; o < 9; ++o) a[o] = __ldg(B + (i64)(9 * z + o) * n + q);
+#pragma unroll
+      for (int o = 0; o < 9; ++o)
+        xv[o] = a[o] != 0.0 ? __ldg(x + q + ((z - 1) * g.ny + o / 3 - 1) * g.nx + o % 3 - 1) : 0.0;
+#pragma unroll
+      for (int o = 0; o < 9; ++o) {
+        if (a[o] == 0.0) continue;
+        const double p = __dmul_rn(-a[o], xv[o]), pe = fma(-a[o], xv[o], -p);
+        const double t = __dadd_rn(s, p), w = __dsub_rn(t, s);
+        e = __dadd_rn(e, __dadd_rn(__dadd_rn(__dsub_rn(s, __dsub_rn(t, w)), __dsub_rn(p, w)), pe));
+        s = t;
+      }
     }
     r[q] = __dadd_rn(s, e);
   }
