@@ -18,9 +18,9 @@
 // term and in the same order: results are theirs bit for bit.  (The __f*_rn
 // intrinsics keep the compiler from contracting what it leaves apart there.)
 //
-// What bounds it: latency at 16 warps per SM (issuing on 45 to 57% of the cycles,
-// DRAM at 43 to 64%).  257^3, the two single passes and the sweep: zero-guess step
-// + residual 142 -> 101 us, two steps 164 -> 119 us with b.z and 138 -> 104 us
+// What bounds it: latency at 16 warps per SM (issuing on 43 to 58% of the cycles,
+// DRAM at 52 to 65%).  257^3, the two single passes and the sweep: zero-guess step
+// + residual 142 -> 100 us, two steps 164 -> 119 us with b.z and 138 -> 104 us
 // (Richardson) without; 513^3: 914 -> 710 us, 1066 -> 1005 us.  Reading the stored
 // 1 / D for the steps instead of dividing: 124 -> 119 us (the same value).  640 and 768 threads
 // per block, at 96 and 80 registers: 161 and 205 us.
