@@ -723,10 +723,10 @@ mg_status read_scal(mg_handle* h);
 // kernel's).  Above, a V-cycle with sweeps and with single passes, float32 / Richardson(8) /
 // bfloat16 coefficients, us: 161^3 vertices 220 : 243 / 561 : 608 / 238 : 265, 193^3 304 : 335 /
 // 769 : 862 / 315 : 355, 257^3 525 : 602 / 1315 : 1545 / 556 : 606, 289^3 797 : 903 / 2111 : 2449 /
-// 848 : 956, 513^3 3561 : 3887 / 9640 : 10275 / 3817 : 3852; 129 x 129 x 273, 321 x 161 x 161 and
-// 81 x 81 x 705 alike in any order of the axes.  The share of points on tile rims (1.94 times the
-// points at 161^3, 1.35 at 257^3, 1.57 at 289^3 and 385^3) does not order these; the one loss found is
-// bfloat16 at 385^3 (1797 : 1774).
+// 848 : 956, 513^3 3561 : 3887 / 9640 : 10275 / 3817 : 3852; boxes from 129 x 129 x 273 to 577 x 577 x 321
+// and 65 x 65 x 1793 alike in any order of the axes.  The share of points on tile rims (1.94 times the
+// points at 161^3, 1.35 at 257^3, 1.57 at 289^3 and 385^3) does not order these; the losses found are
+// bfloat16 at 385^3 (1797 : 1774) and 385 x 257 x 513 (1563 : 1553).
 constexpr double PAIR_MIN_POINTS = 4e6;
 
 template <class TV, class TC> struct Impl {
